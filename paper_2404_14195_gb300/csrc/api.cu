@@ -592,7 +592,7 @@ int compute_weights_impl(rbf_ctx *ctx, int phs_k, int mono_m, int solver, int q,
     if (!presolved) {
         CK(ctx->w64.alloc(n * n_ops * n_l));
         CK(ctx->delta.alloc(n));
-        CK(launch_weights(n, ctx->xyz.p, nullptr, ctx->iota.p, 1, n_l, ctx->idx.p, phs_k, mono_m, n_ops, d_ops.p, 1,
+        CK(launch_weights(n, ctx->xyz.p, nullptr, ctx->iota.p, 1, n_l, ctx->idx.p, phs_k, mono_m, n_ops, d_ops.p,
                           ctx->w64.p, ctx->delta.p, ctx->status.p, ctx->st));
         ++ctx->launches;
         CK(ctx->wgb64.alloc(nb * 3 * n_l));
@@ -604,9 +604,9 @@ int compute_weights_impl(rbf_ctx *ctx, int phs_k, int mono_m, int solver, int q,
             ++ctx->launches;
             if (!presolved)
                 CK(launch_weights(nb, ctx->xyz.p, nullptr, ctx->wall.p, 1, n_l, ctx->idxb.p, phs_k, mono_m, 3, d_gops.p,
-                                  1, ctx->wgb64.p, nullptr, ctx->status.p + 1, ctx->st));
+                                  ctx->wgb64.p, nullptr, ctx->status.p + 1, ctx->st));
         } else {
-            CK(launch_weights(nb, ctx->xyz.p, nullptr, ctx->wall.p, 1, n_l, ctx->idxw.p, phs_k, mono_m, 3, d_gops.p, 1,
+            CK(launch_weights(nb, ctx->xyz.p, nullptr, ctx->wall.p, 1, n_l, ctx->idxw.p, phs_k, mono_m, 3, d_gops.p,
                               ctx->wgw64.p, nullptr, ctx->status.p + 1, ctx->st));
         }
         ++ctx->launches;
@@ -1195,7 +1195,7 @@ int ensure_probes(rbf_ctx *ctx, int m_p) {
         CK(d_op.alloc(1));
         CK(cudaMemcpyAsync(d_op.p, &op, sizeof(OpSpec), cudaMemcpyHostToDevice, ctx->st));
         CK(launch_weights(nfl, ctx->xyz.p, pxyz.p, nullptr, 0, n_l, pidx.p, ctx->phs_k, ctx->mono_m, 1,
-                          d_op.p, 1, pw.p, nullptr, ctx->status.p + 1, ctx->st));
+                          d_op.p, pw.p, nullptr, ctx->status.p + 1, ctx->st));
         ctx->launches += 2;
     }
     int32_t st2[2] = {0, 0};
@@ -1727,12 +1727,12 @@ int rbf_batch_build(rbf_batch *b, int phs_k, int mono_m, rbf_weight_report *rep)
     CK(cudaMemcpyAsync(dops.p, ops.data(), 4 * sizeof(OpSpec), cudaMemcpyHostToDevice, b->st));
     CK(cudaMemcpyAsync(dgops.p, gops.data(), 3 * sizeof(OpSpec), cudaMemcpyHostToDevice, b->st));
     CK(dsing.zero(b->st));
-    CK(launch_weights_multi(nc, dj.p, dpn.p, pn[nc], max_nl, phs_k, mono_m, 4, dops.p, 1, dsing.p, b->st));
+    CK(launch_weights_multi(nc, dj.p, dpn.p, pn[nc], max_nl, phs_k, mono_m, 4, dops.p, dsing.p, b->st));
     if (!walls.empty()) {
         CK(dwj.alloc(walls.size())); CK(dpw.alloc(pw.size()));
         CK(cudaMemcpyAsync(dwj.p, walls.data(), walls.size() * sizeof(WeightJob), cudaMemcpyHostToDevice, b->st));
         CK(cudaMemcpyAsync(dpw.p, pw.data(), pw.size() * sizeof(int64_t), cudaMemcpyHostToDevice, b->st));
-        CK(launch_weights_multi((int)walls.size(), dwj.p, dpw.p, pw.back(), max_nl, phs_k, mono_m, 3, dgops.p, 1,
+        CK(launch_weights_multi((int)walls.size(), dwj.p, dpw.p, pw.back(), max_nl, phs_k, mono_m, 3, dgops.p,
                                 dsing.p + 1, b->st));
     }
     int32_t sing[2] = {0, 0};
