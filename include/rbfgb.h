@@ -302,13 +302,16 @@ int rbf_autotune(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep);
  * only; 2 <= trial_steps <= 20000.  rep->code[c] is the code of candidate c. */
 int rbf_autotune_persistent(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep);
 /* Schedule of the persistent ACM driver for this context, as a code:
- *   block + 1000 G   a cooperative grid of `block` (32, 64, 128, 256; default 256)
- *                    threads per block whose sweeps give each node G lanes (2, 4
- *                    or 8; write 0 for G = 1, i.e. the code is the block size):
- *                    the lanes split the node's stencil columns and combine their
- *                    partial sums with shuffles, multiplying the warps at work on
- *                    small cells;
+ *   block + 1000 G   a cooperative grid of `block` (32, 64, 128, 256) threads per
+ *                    block whose sweeps give each node G lanes (2, 4 or 8; write 0
+ *                    for G = 1, i.e. the code is the block size): the lanes split
+ *                    the node's stencil columns and combine their partial sums
+ *                    with shuffles, multiplying the warps at work on small cells.
+ *                    With G > 1 a single cell whose stencils fit the SMs' shared
+ *                    memory runs resident there, one block of at least 256
+ *                    threads per SM;
  *   -8, -16          one cluster of 8 / 16 CTAs of 256 threads, G = 1.
+ * Until a code is set the schedule is chosen by the size of the cells.
  * A batch launches with its first cell's setting.  With G = 1 the schedule
  * changes only the order of the FP64 residual partial sums; G > 1 also changes
  * the order of the stencil sums (rounding only). */

@@ -30,31 +30,51 @@ struct CellDesc {
 };
 
 struct PersistCtl {
-    unsigned *bar_count, *bar_gen;
+    unsigned *bar;           // barrier words (acm_persist.cu), zero at launch, 256 bytes
     int32_t *err;            // 2 = a grid barrier timed out
     int32_t *done;           // per cell: 0 running, 1 converged, 3 non-finite residual
     int64_t *steps;          // per cell: steps taken in this launch
     double *resid;           // per cell: last residual
     double *partial;         // [block][PERSIST_MAX_CELLS][2]
     int ncells;
-    int64_t nslices, nwslices;
-    const int2 *slices;      // (cell, slice within the cell) of every node slice
-    const int2 *wslices;     // the same for the wall lists
     int64_t max_steps;
     int check_every;
     double tol;
     int n_p;
     uint64_t wait_ns;        // wall-clock limit of one grid-barrier wait (nanoseconds)
+    unsigned long long *vsq; // resident kernel: 2 slots of max |v|^2
 };
 
+// shared memory of the streaming kernel: descriptors, residual accumulators, unit
+// counts ahead of each cell, flags
+template <typename T>
+__host__ __device__ constexpr int64_t persist_head_bytes(int ncells) {
+    return ((int64_t)ncells * (int64_t)sizeof(CellDesc<T>) + (ncells + 1) * 16ll + ncells * 16ll + ncells * 4ll + 15) & ~15ll;
+}
+// Shares of the resident kernel (one cell, every block's stencils in shared memory):
+// largest number of units and wall units per block, local nodes there is room for,
+// dynamic shared memory, blocks.
+struct ResPlan {
+    int units, wunits, loc, smem, nblocks;
+};
+// whether a cell can run resident with `room` bytes of shared memory on each of `sms` SMs (its
+// local sets are only known to the kernel, which raises error 3 before the first step if one has
+// no room)
+template <typename T>
+bool acm_resident_plan(int64_t n, int64_t nb, int n_l, int group, int sms, int64_t room, ResPlan *pl);
+template <typename T>
+cudaError_t acm_launch_resident(const CellDesc<T> &cell, const PersistCtl &ctl, const ResPlan &pl, int block, int group,
+                                bool cp, cudaStream_t st);
+
 // cp selects the compensated kernel (every cell then carries low words); block:
-// threads per block, 32, 64, 128 or 256; group: lanes per node, 1, 2, 4 or 8 (a
-// warp takes 32 / group nodes of a slice at a time)
+// threads per block, 32, 64, 128 or 256; group: lanes per node,
+// 1, 2, 4 or 8 (a warp takes 32 / group nodes of a slice at a time)
 template <typename T>
 cudaError_t acm_launch_persistent(const CellDesc<T> *cells_dev, const PersistCtl &ctl, int nblocks, int block,
                                   int group, bool cp, cudaStream_t st);
+// co-resident blocks of the kernel with `smem` bytes of dynamic shared memory each
 template <typename T>
-cudaError_t acm_persistent_max_blocks(int *blocks, int block, int group, bool cp);
+cudaError_t acm_persistent_max_blocks(int *blocks, int block, int group, bool cp, size_t smem);
 // the same kernel as one thread-block cluster of csize (8 or 16) CTAs of 256
 // threads, synchronised by the cluster barrier
 template <typename T>
@@ -62,6 +82,6 @@ cudaError_t acm_launch_persistent_cluster(const CellDesc<T> *cells_dev, const Pe
                                           cudaStream_t st);
 // whether a cluster of csize CTAs of the kernel can be scheduled on this device
 template <typename T>
-cudaError_t acm_persistent_cluster_ok(int csize, bool cp, bool *ok);
+cudaError_t acm_persistent_cluster_ok(int csize, bool cp, size_t smem, bool *ok);
 
 }  // namespace rbf

@@ -84,6 +84,18 @@ cudaError_t lbm_macro_current(rbf_ctx *c) {
 
 int persistent_solve(std::vector<rbf_ctx *> &cs, const rbf_solve_opts *o, std::vector<int64_t> &steps,
                      std::vector<double> &resid, std::vector<int32_t> &done, std::string &err);
+// Schedule of the resident ACM driver when none was set, from the nodes per SM: more lanes
+// per node shorten the serial sums, fewer do less work in the combination.  Measured
+// (us per step at N_L = 25, lanes 1 / 2 / 4 / 8, 256-512 threads):
+//   FP32  15 nodes per SM 29 / 25 / 24 / 24, 44: 31 / 26 / 26 / 29, 86: 32 / 27 / 29 / 34,
+//         163: 33.6 / 31.8 / 36 / 40, 276: 37 / 39 / 42 / 51
+//   FP64  15: 58 / 42 / 34 / 34, 44: 59 / 43 / 39 / 52, 86: 60 / 49 / 52 / 79,
+//         163: 70 / 70 / 80 / 129
+// Blocks of 1024 threads cost 2 us more per step.
+void resident_auto(double per_sm, bool fp64, int *block, int *group) {
+    *group = per_sm <= 60.0 ? 4 : (per_sm <= (fp64 ? 160.0 : 200.0) ? 2 : 1);
+    *block = per_sm <= 60.0 ? 256 : 512;
+}
 cudaError_t static_flux_lookup(double **out);
 
 void drop_graph(rbf_ctx *ctx) {
@@ -494,6 +506,7 @@ int rbf_build_stencils(rbf_ctx *ctx, int n_l) {
     drop_graph(ctx);
     ctx->weights_ok = false;
     ctx->inited = false;
+    ctx->res_nofit = false;
     ctx->m_p = 0;
     const int64_t n = ctx->n;
     int G = (int)std::lround(std::cbrt((double)n / 4.0));
@@ -977,8 +990,9 @@ int tune_persistent(std::vector<rbf_ctx *> &cs, int trial_steps, rbf_tune_report
     std::vector<int> cands = {256, 128, 64, 32, 2128, 4128, 8128, 4256};
     for (int c : {16, 8}) {
         bool ok = false;
-        if (is_f32(ctx)) CK(acm_persistent_cluster_ok<float>(c, ctx->prec == RBF_FP32C, &ok));
-        else CK(acm_persistent_cluster_ok<double>(c, false, &ok));
+        const int nc = (int)cs.size();
+        if (is_f32(ctx)) CK(acm_persistent_cluster_ok<float>(c, ctx->prec == RBF_FP32C, (size_t)persist_head_bytes<float>(nc), &ok));
+        else CK(acm_persistent_cluster_ok<double>(c, false, (size_t)persist_head_bytes<double>(nc), &ok));
         if (ok) cands.push_back(-c);
     }
     rbf_tune_report r;
@@ -1346,6 +1360,68 @@ int rbf_pointwise_difference(rbf_ctx *a, rbf_ctx *b, double *delta, double *dv) 
 
 namespace {
 
+// Grid and schedule of a persistent launch over `cs`.
+struct PersistPlan {
+    cudaError_t err = cudaSuccess;
+    int csize = 0, nblocks = 1, block = 256, group = 1;
+    bool resident = false;
+    ResPlan res{};
+};
+template <typename T>
+PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
+    PersistPlan p;
+    const rbf_ctx *x = cs[0];
+    if (x->persist_cluster) {
+        p.csize = p.nblocks = x->persist_cluster;
+        return p;
+    }
+    int sms = 0, optin = 0;
+    p.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, x->device);
+    if (p.err == cudaSuccess) p.err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, x->device);
+    if (p.err != cudaSuccess) return p;
+    // One cell whose shares fit runs resident, unless one lane per node was asked for (which
+    // keeps the summation order of the multi-launch kernels).
+    if (cs.size() == 1 && !x->res_nofit && (!x->persist_block || x->persist_group > 1)) {
+        p.group = x->persist_group;
+        if (!x->persist_block) resident_auto(x->n / (double)sms, sizeof(T) == 8, &p.block, &p.group);
+        else p.block = std::min<int>(sizeof(T) == 4 ? 1024 : 512, std::max<int>(x->persist_block, 256));
+        p.resident = acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, sms, optin - 2048, &p.res);
+        if (p.resident) {
+            p.nblocks = p.res.nblocks;
+            return p;
+        }
+    }
+    int64_t slices = 0;
+    for (const rbf_ctx *y : cs) slices += y->npad / 32;
+    // blocks and the share of the last round's warps that have a unit
+    auto grid = [&](int block, int group, int *nblocks) -> double {
+        int maxb = 0;
+        p.err = acm_persistent_max_blocks<T>(&maxb, block, group, cp, (size_t)persist_head_bytes<T>((int)cs.size()));
+        const int64_t wpb = block / 32, units = slices * group;
+        *nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(maxb, (units + wpb - 1) / wpb));
+        const double rounds = (double)units / ((double)*nblocks * wpb);
+        return rounds / std::ceil(rounds);
+    };
+    if (x->persist_block) {
+        p.block = x->persist_block;
+        p.group = x->persist_group;
+        grid(p.block, p.group, &p.nblocks);
+        return p;
+    }
+    // One lane per node, unless that leaves the last round of units so empty that two lanes per
+    // node, 8 % slower per unit, finish earlier (485k nodes in 12 cells: 3.1 rounds, 506 us per
+    // step against 484 with two lanes; 600k nodes: 3.9 rounds, 568 against 652)
+    int nb1 = 1, nb2 = 1;
+    const double e1 = grid(256, 1, &nb1);
+    if (p.err != cudaSuccess) return p;
+    const double e2 = grid(128, 2, &nb2);
+    const bool two = 0.92 * e2 > e1;
+    p.block = two ? 128 : 256;
+    p.group = two ? 2 : 1;
+    p.nblocks = two ? nb2 : nb1;
+    return p;
+}
+
 // Steady ACM solve of one or more initialised contexts (same device, stream,
 // precision and n_p) in one persistent cooperative launch.  Per cell: steps taken,
 // last residual, status (1 converged, 0 step cap, 3 non-finite).
@@ -1355,7 +1431,6 @@ int persistent_solve_T(std::vector<rbf_ctx *> &cs, cudaStream_t st, const rbf_so
     rbf_ctx *ctx = cs[0];  // for CK's error reporting
     const int nc = (int)cs.size();
     std::vector<CellDesc<T>> desc(nc);
-    std::vector<int2> sl, wsl;
     for (int c = 0; c < nc; ++c) {
         rbf_ctx *x = cs[c];
         DevArr<T> *a = nullptr;
@@ -1377,44 +1452,34 @@ int persistent_solve_T(std::vector<rbf_ctx *> &cs, cudaStream_t st, const rbf_so
         }
         d.dt = (T)x->dt; d.nu = (T)x->prm.nu; d.gx = (T)x->prm.g[0]; d.gy = (T)x->prm.g[1]; d.gz = (T)x->prm.g[2];
         d.rho = (T)x->rho; d.beta = x->beta; d.vref = x->vref;
-        for (int64_t s = 0; s < x->npad / 32; ++s) sl.push_back(make_int2(c, (int)s));
-        for (int64_t s = 0; s < (x->nb + 31) / 32; ++s) wsl.push_back(make_int2(c, (int)s));
     }
     const bool cp = cs[0]->prec == RBF_FP32C;
-    const int csize = cs[0]->persist_cluster;
-    const int block = csize ? 256 : cs[0]->persist_block, wpb = block / 32;
-    const int group = csize ? 1 : cs[0]->persist_group;
-    int nblocks = csize;
-    if (!csize) {
-        int maxb = 0;
-        CK(acm_persistent_max_blocks<T>(&maxb, block, group, cp));
-        const int64_t units = (int64_t)sl.size() * group;  // work units of 32 / group nodes
-        nblocks = std::max(1, std::min<int>(maxb, (int)((units + wpb - 1) / wpb)));
-    }
-    DevArr<CellDesc<T>> d_desc;
-    DevArr<int2> d_sl, d_wsl;
-    DevArr<unsigned> d_bar;
-    DevArr<int32_t> d_err, d_done;
-    DevArr<int64_t> d_steps;
-    DevArr<double> d_res, d_part;
-    CK(d_desc.alloc(nc)); CK(d_sl.alloc(sl.size())); CK(d_wsl.alloc(std::max<size_t>(wsl.size(), 1)));
-    CK(d_bar.alloc(2)); CK(d_err.alloc(1)); CK(d_done.alloc(nc)); CK(d_steps.alloc(nc)); CK(d_res.alloc(nc));
-    CK(d_part.alloc((size_t)nblocks * 2 * PERSIST_MAX_CELLS));
-    CK(cudaMemcpyAsync(d_desc.p, desc.data(), nc * sizeof(CellDesc<T>), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(d_sl.p, sl.data(), sl.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
-    if (!wsl.empty()) CK(cudaMemcpyAsync(d_wsl.p, wsl.data(), wsl.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
-    CK(d_bar.zero(st)); CK(d_err.zero(st)); CK(d_done.zero(st)); CK(d_steps.zero(st)); CK(d_res.zero(st));
+    const PersistPlan pl = persist_plan<T>(cs, cp);
+    if (pl.err != cudaSuccess) return cuda_fail(ctx, pl.err, "persistent driver plan");
+    // one workspace, kept by the first cell: descriptors, then what the kernel clears from
+    // (barrier counter, error flag, done, steps, residuals), then the block partials
+    const size_t o_desc = 0, o_bar = (nc * sizeof(CellDesc<T>) + 255) & ~(size_t)255, o_done = o_bar + 256 + 32;
+    const size_t o_steps = o_done + ((nc * 4 + 15) & ~(size_t)15), o_res = o_steps + nc * 8, o_part = (o_res + nc * 8 + 255) & ~(size_t)255;
+    const size_t need = o_part + (size_t)pl.nblocks * 2 * PERSIST_MAX_CELLS * sizeof(double);
+    if (ctx->persist_ws.n < need) CK(ctx->persist_ws.alloc(need));
+    char *ws = ctx->persist_ws.p;
+    if (!pl.resident) CK(cudaMemcpyAsync(ws + o_desc, desc.data(), nc * sizeof(CellDesc<T>), cudaMemcpyHostToDevice, st));
+    CK(cudaMemsetAsync(ws + o_bar, 0, o_part - o_bar, st));
     PersistCtl ctl;
     std::memset(&ctl, 0, sizeof(ctl));
-    ctl.bar_count = d_bar.p; ctl.bar_gen = d_bar.p + 1; ctl.err = d_err.p; ctl.done = d_done.p; ctl.steps = d_steps.p;
-    ctl.resid = d_res.p; ctl.partial = d_part.p; ctl.ncells = nc; ctl.nslices = (int64_t)sl.size();
-    ctl.nwslices = (int64_t)wsl.size(); ctl.slices = d_sl.p; ctl.wslices = d_wsl.p; ctl.max_steps = o->max_steps;
+    ctl.bar = (unsigned *)(ws + o_bar); ctl.err = (int32_t *)(ws + o_bar + 256); ctl.done = (int32_t *)(ws + o_done);
+    ctl.steps = (int64_t *)(ws + o_steps); ctl.resid = (double *)(ws + o_res); ctl.partial = (double *)(ws + o_part);
+    ctl.ncells = nc; ctl.max_steps = o->max_steps;
     ctl.check_every = o->check_every > 0 ? o->check_every : 100; ctl.tol = o->tol; ctl.n_p = cs[0]->n_p;
-    ctl.wait_ns = cs[0]->wait_ns;
+    ctl.wait_ns = cs[0]->wait_ns; ctl.vsq = (unsigned long long *)(ws + o_bar + 256 + 16);
+    const CellDesc<T> *d_desc = (const CellDesc<T> *)(ws + o_desc);
     CK(cudaEventRecord(ctx->ev0, st));
-    if (csize) CK(acm_launch_persistent_cluster<T>(d_desc.p, ctl, csize, cp, st));
-    else CK(acm_launch_persistent<T>(d_desc.p, ctl, nblocks, block, group, cp, st));
+    if (pl.resident) CK(acm_launch_resident<T>(desc[0], ctl, pl.res, pl.block, pl.group, cp, st));
+    else if (pl.csize) CK(acm_launch_persistent_cluster<T>(d_desc, ctl, pl.csize, cp, st));
+    else CK(acm_launch_persistent<T>(d_desc, ctl, pl.nblocks, pl.block, pl.group, cp, st));
     CK(cudaEventRecord(ctx->ev1, st));
+    std::vector<char> back(o_part - o_bar);
+    CK(cudaMemcpyAsync(back.data(), ws + o_bar, back.size(), cudaMemcpyDeviceToHost, st));
     for (rbf_ctx *x : cs) x->launches += 1;
     CK(cudaStreamSynchronize(st));
     {
@@ -1424,13 +1489,17 @@ int persistent_solve_T(std::vector<rbf_ctx *> &cs, cudaStream_t st, const rbf_so
     }
     int32_t e = 0;
     steps.assign(nc, 0); resid.assign(nc, 0.0); done.assign(nc, 0);
-    CK(cudaMemcpy(&e, d_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(steps.data(), d_steps.p, nc * sizeof(int64_t), cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(resid.data(), d_res.p, nc * sizeof(double), cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(done.data(), d_done.p, nc * sizeof(int32_t), cudaMemcpyDeviceToHost));
+    std::memcpy(&e, back.data() + 256, sizeof(e));
+    std::memcpy(done.data(), back.data() + (o_done - o_bar), nc * sizeof(int32_t));
+    std::memcpy(steps.data(), back.data() + (o_steps - o_bar), nc * sizeof(int64_t));
+    std::memcpy(resid.data(), back.data() + (o_res - o_bar), nc * sizeof(double));
     for (int c = 0; c < nc; ++c) {
         cs[c]->parity = (int)((cs[c]->parity + (int64_t)cs[c]->n_p * steps[c]) & 1);
         drop_graph(cs[c]);
+    }
+    if (e == 3) {  // no step was taken: a share's local node set has no room
+        ctx->res_nofit = true;
+        return persistent_solve_T<T>(cs, st, o, steps, resid, done, err);
     }
     if (e) {
         err = "persistent ACM driver: a grid barrier timed out";

@@ -95,15 +95,17 @@ struct rbf_ctx {
     // scratch
     DevArr<double> partial, scal, mac, stage;  // stage: host <-> device field transfers
     DevArr<int32_t> status;
+    DevArr<char> persist_ws;  // descriptors and control words of the persistent ACM driver
     // graph of `gsteps` steps
     cudaGraphExec_t gexec = nullptr;
     int gsteps = 0, gparity = -1, gcur = -1, gprec = -1, gvariant = -1, gphase = -1;
     int variant = rbf::LBM_PAIR_PER_WARP;  // schedule of the fused LBM step
     int lbm_layout = rbf::LBM_LAYOUT_PAIRS;  // layout of f32 / f64 (follows the schedule)
     int acm_code = 256;               // ACM sweeps: threads per block + 1000 x lanes per node (0: one)
-    int persist_block = 256;          // threads per block of the persistent ACM driver
+    int persist_block = 0;            // threads per block of the persistent ACM driver (0: chosen by size)
     int persist_cluster = 0;          // > 0: run it as one cluster of that many CTAs (8 or 16)
     int persist_group = 1;            // lanes per node of its sweeps (1, 2, 4, 8)
+    bool res_nofit = false;           // a share's local nodes did not fit the resident driver (these stencils)
     double persist_ms = 0.0;          // device time of its last launch
     uint64_t wait_ns = 2000000000ull; // wall-clock limit of one grid-barrier wait of that driver
     int gblock = -1;
