@@ -253,16 +253,19 @@ int rbf_profile_steps(rbf_ctx *ctx, int nsteps, double *kernel_ms, int *n_classe
 /* Schedule of the fused LBM step (all compute the same step; only the thread
  * mapping and the population layout differ): 0 one node per thread, 256-thread
  * blocks; 1 one opposite-population pair per warp, (q-1)/2 warps per 32-node
- * slice, moments reduced in shared memory, stencil loop unrolled 5 deep
- * (default); 2 as 0 with 128-thread blocks; 3, 4, 5 as 1 unrolled 3, 6, 2 deep.
+ * slice, moments reduced in shared memory, stencil loop unrolled 5 deep;
+ * 2 as 0 with 128-thread blocks; 3, 4, 5 as 1 unrolled 3, 6, 2 deep.
  * 0-5 keep the populations as the rest population plus interleaved opposite
- * pairs; 6 and 7 keep each node's q populations in one record of q rounded up
- * to a multiple of 4 values, read with 16-byte loads: 6 one node per thread,
- * 256-thread blocks; 7 the same with registers capped so that five blocks fit
- * on an SM; 8 and 9 as 6 in blocks of 128 and 64 threads (finer blocks spread
- * the nodes more evenly over the SMs); 10 as 6, launched as a programmatic
- * dependent launch (the next step's blocks are scheduled while this step drains
- * and wait on the grid dependency before touching memory).  Switching between the two layouts on an initialised LBM
+ * pairs; 6 to 10 keep each node's q populations in one record of q rounded up
+ * to a multiple of 4 values, read with 16-byte loads: 6 one node per thread
+ * (small cells: 2, 4 or 8 lanes per node, which split its stencil columns),
+ * 256-thread blocks; 7 one node per thread with registers capped so that more
+ * blocks fit on an SM; 8 and 9 as 6 in blocks of 128 and 64 threads; 10 as 6 with
+ * blocks by the size of the grid, a grid that fills the chip launched as a
+ * programmatic dependent launch (the next step's blocks are scheduled while this
+ * step drains and wait on the grid dependency before touching memory).  Until a
+ * code is set: 10, cells below 4096 nodes 1.
+ * Switching between the two layouts on an initialised LBM
  * context rewrites the state (one kernel launch); the populations, as
  * rbf_lbm_get_populations reports them, are unchanged.
  * On a context whose weights were computed for RBF_SOLVER_ACM the code selects the

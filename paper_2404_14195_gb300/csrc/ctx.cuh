@@ -43,7 +43,7 @@ struct DevArr {
 
 struct rbf_ctx {
     template <typename T> using DevArr = rbf::DevArr<T>;
-    int device = 0;
+    int device = 0, sms = 1;
     cudaStream_t st = nullptr;
     bool own_stream = false;
     std::string err;
@@ -99,8 +99,9 @@ struct rbf_ctx {
     // graph of `gsteps` steps
     cudaGraphExec_t gexec = nullptr;
     int gsteps = 0, gparity = -1, gcur = -1, gprec = -1, gvariant = -1, gphase = -1;
-    int variant = rbf::LBM_PAIR_PER_WARP;  // schedule of the fused LBM step
-    int lbm_layout = rbf::LBM_LAYOUT_PAIRS;  // layout of f32 / f64 (follows the schedule)
+    int variant = rbf::LBM_RECORD_PER_THREAD_PDL;  // schedule of the fused LBM step
+    bool variant_auto = true;                      // not set by the caller: chosen by size in rbf_init
+    int lbm_layout = rbf::LBM_LAYOUT_NODES;  // layout of f32 / f64 (follows the schedule)
     int acm_code = 256;               // ACM sweeps: threads per block + 1000 x lanes per node (0: one)
     int persist_block = 0;            // threads per block of the persistent ACM driver (0: chosen by size)
     int persist_cluster = 0;          // > 0: run it as one cluster of that many CTAs (8 or 16)

@@ -24,23 +24,50 @@
 namespace rbf {
 
 // Velocity sets in the paper's convention: odd k listed, e_k = -e_{k-1} for even k.
-// D3Q15 as tabulated in the MLBM section; D3Q19 with the textbook weights.
-__constant__ int c_e15[15][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
-                                 {0, 0, 1},  {0, 0, -1}, {1, 1, 1},  {-1, -1, -1}, {1, 1, -1},
-                                 {-1, -1, 1}, {1, -1, 1}, {-1, 1, -1}, {1, -1, -1}, {-1, 1, 1}};
-__constant__ int c_e19[19][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0}, {0, 0, 1},  {0, 0, -1},
-                                 {1, 1, 0},  {-1, -1, 0}, {1, -1, 0}, {-1, 1, 0}, {1, 0, 1},  {-1, 0, -1},
-                                 {1, 0, -1}, {-1, 0, 1}, {0, 1, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
-
+// D3Q15 as tabulated in the MLBM section; D3Q19 with the textbook weights.  The
+// components are compile-time constants in unrolled code, so a moment is additions
+// only: no products with 0 and +-1, which in FP64 cost as much as any other.
 template <int Q> struct VSet;
 template <> struct VSet<19> {
     static __host__ __device__ constexpr double w(int k) { return k == 0 ? 1.0 / 3.0 : (k <= 6 ? 1.0 / 18.0 : 1.0 / 36.0); }
-    static __device__ __forceinline__ int e(int k, int a) { return c_e19[k][a]; }
+    static __host__ __device__ constexpr int e(int k, int a) {
+        constexpr int t[19][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0}, {0, 0, 1},  {0, 0, -1},
+                                  {1, 1, 0},  {-1, -1, 0}, {1, -1, 0}, {-1, 1, 0}, {1, 0, 1},  {-1, 0, -1},
+                                  {1, 0, -1}, {-1, 0, 1}, {0, 1, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
+        return t[k][a];
+    }
 };
 template <> struct VSet<15> {
     static __host__ __device__ constexpr double w(int k) { return k == 0 ? 2.0 / 9.0 : (k <= 6 ? 1.0 / 9.0 : 1.0 / 72.0); }
-    static __device__ __forceinline__ int e(int k, int a) { return c_e15[k][a]; }
+    static __host__ __device__ constexpr int e(int k, int a) {
+        constexpr int t[15][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
+                                  {0, 0, 1},  {0, 0, -1}, {1, 1, 1},  {-1, -1, -1}, {1, 1, -1},
+                                  {-1, -1, 1}, {1, -1, 1}, {-1, 1, -1}, {1, -1, -1}, {-1, 1, 1}};
+        return t[k][a];
+    }
 };
+// the same table for a k known only at run time
+__constant__ signed char c_e19[19][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},  {0, -1, 0}, {0, 0, 1},  {0, 0, -1},
+                                         {1, 1, 0},  {-1, -1, 0}, {1, -1, 0}, {-1, 1, 0}, {1, 0, 1},  {-1, 0, -1},
+                                         {1, 0, -1}, {-1, 0, 1}, {0, 1, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
+__constant__ signed char c_e15[15][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
+                                         {0, 0, 1},  {0, 0, -1}, {1, 1, 1},  {-1, -1, -1}, {1, 1, -1},
+                                         {-1, -1, 1}, {1, -1, 1}, {-1, 1, -1}, {1, -1, -1}, {-1, 1, 1}};
+template <int Q>
+__device__ __forceinline__ int c_e(int k, int a) { return Q == 15 ? c_e15[k % 15][a] : c_e19[k][a]; }
+// s + e x for a velocity component e = -1, 0 or 1 known at compile time
+template <typename T>
+__device__ __forceinline__ T add_e(T s, int e, T x) { return e == 0 ? s : (e > 0 ? s + x : s - x); }
+// e . (x, y, z)
+template <int Q, typename T>
+__device__ __forceinline__ T dot_e(int k, T x, T y, T z) {
+    T s = (T)0;
+    bool first = true;
+    if (VSet<Q>::e(k, 0)) { s = VSet<Q>::e(k, 0) > 0 ? x : -x; first = false; }
+    if (VSet<Q>::e(k, 1)) { s = first ? (VSet<Q>::e(k, 1) > 0 ? y : -y) : add_e(s, VSet<Q>::e(k, 1), y); first = false; }
+    if (VSet<Q>::e(k, 2)) { s = first ? (VSet<Q>::e(k, 2) > 0 ? z : -z) : add_e(s, VSet<Q>::e(k, 2), z); }
+    return s;
+}
 
 const int *host_velocity_set(int q) {
     static const int e15[15][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
@@ -73,6 +100,7 @@ __global__ void k_lbm_masks(int64_t n, const uint8_t *__restrict__ type, const d
     if (i >= n) return;
     uint32_t m = 0;
     if (type[i]) {
+#pragma unroll
         for (int k = 1; k < Q; ++k) {
             double en = __dadd_rn(__dadd_rn(__dmul_rn((double)VSet<Q>::e(k, 0), nrm[3 * i]),
                                             __dmul_rn((double)VSet<Q>::e(k, 1), nrm[3 * i + 1])),
@@ -97,8 +125,10 @@ __global__ void k_lbm_masks_solid(int64_t n, const uint8_t *__restrict__ type, c
     if (type[i]) {
         const double c[3] = {c0, c1, c2};
         const double r2 = __dmul_rn(r, r);
+#pragma unroll
         for (int k = 1; k < Q; ++k) {
             double d[3];
+#pragma unroll
             for (int a = 0; a < 3; ++a) {
                 const double p = __dsub_rn(xyz[3 * i + a], __dmul_rn(dx, (double)VSet<Q>::e(k, a)));
                 const double v = __dsub_rn(p, c[a]);
@@ -111,19 +141,32 @@ __global__ void k_lbm_masks_solid(int64_t n, const uint8_t *__restrict__ type, c
     mask[i] = m;
 }
 
-// TRT collision of one node in shifted variables; f[] in, f[] out (post-collision)
+// a / b, b near 1, for several a: FP64 from one reciprocal r = 1 / b and a residual
+// correction each (a division is some twenty operations on the pipe that bounds the step)
+__device__ __forceinline__ float over(float a, float b, float) { return a / b; }
+__device__ __forceinline__ double over(double a, double b, double r) {
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
+}
+
+// TRT collision of one node in shifted variables; f[] in, f[] out (post-collision).  The
+// non-equilibrium parts are formed as differences before they are scaled: near the steady
+// state populations and equilibria nearly cancel, and scaling the two sides apart leaves
+// the rounding of the two factors as a bias in every step (measured: 3.5 times the error
+// against 64-bit references after 100 steps).
 template <typename T, int Q>
 __device__ __forceinline__ void trt_collide(T (&f)[Q], T tp_inv, T tm_inv, T gx, T gy, T gz) {
-    T drho = 0, mx = 0, my = 0, mz = 0;
+    T drho = f[0], mx = 0, my = 0, mz = 0;
 #pragma unroll
-    for (int k = 0; k < Q; ++k) {
+    for (int k = 1; k < Q; ++k) {
         drho += f[k];
-        mx += (T)VSet<Q>::e(k, 0) * f[k];
-        my += (T)VSet<Q>::e(k, 1) * f[k];
-        mz += (T)VSet<Q>::e(k, 2) * f[k];
+        mx = add_e(mx, VSet<Q>::e(k, 0), f[k]);
+        my = add_e(my, VSet<Q>::e(k, 1), f[k]);
+        mz = add_e(mz, VSet<Q>::e(k, 2), f[k]);
     }
     const T rho = (T)1 + drho;
-    const T vx = mx / rho, vy = my / rho, vz = mz / rho;
+    const T inv = (T)1 / rho;
+    const T vx = over(mx, rho, inv), vy = over(my, rho, inv), vz = over(mz, rho, inv);
     const T vv = vx * vx + vy * vy + vz * vz;
     const T base = rho * ((T)-1.5 * vv);
     {   // rest population: symmetric only, no force
@@ -134,15 +177,14 @@ __device__ __forceinline__ void trt_collide(T (&f)[Q], T tp_inv, T tm_inv, T gx,
 #pragma unroll
     for (int k = 1; k < Q; k += 2) {
         const T wk = (T)VSet<Q>::w(k);
-        const T ex = (T)VSet<Q>::e(k, 0), ey = (T)VSet<Q>::e(k, 1), ez = (T)VSet<Q>::e(k, 2);
-        const T eu = ex * vx + ey * vy + ez * vz;
+        const T eu = dot_e<Q>(k, vx, vy, vz);
         const T eqp = wk * (drho + base + rho * ((T)4.5 * eu * eu));  // symmetric part of f~_eq
         const T eqm = wk * rho * ((T)3 * eu);                          // antisymmetric part
         const T fp = (T)0.5 * (f[k] + f[k + 1]);
         const T fm = (T)0.5 * (f[k] - f[k + 1]);
         const T dp = (fp - eqp) * tp_inv;
         const T dm = (fm - eqm) * tm_inv;
-        const T F = wk * (T)3 * rho * (ex * gx + ey * gy + ez * gz);
+        const T F = wk * (T)3 * rho * dot_e<Q>(k, gx, gy, gz);
         f[k] = f[k] - dp - dm + F;
         f[k + 1] = f[k + 1] - dp + dm - F;
     }
@@ -223,51 +265,61 @@ template <> struct Vec16<double> {
     static __device__ __forceinline__ double2 make(const double *d) { return make_double2(d[0], d[1]); }
 };
 
-// One thread per node on the node layout: each stencil column costs one index
-// load, (q-1)/2 coalesced 8-byte weight loads and lbm_rec_len(q) / 4 16-byte
-// loads of the neighbour's record (FP32 D3Q19: 5, against 9 pair gathers on the
-// pairs layout).  MINB: blocks of 256 threads the compiler must fit on one SM,
-// i.e. a register cap (FP32: 4 -> 64 registers, no spills; 5 -> 48 registers, a
-// few spills, more warps in flight).  Same arithmetic, in the same order, as
-// k_lbm_step.  PDL: launched as a programmatic dependent of the previous kernel in
-// the stream; every block first lets the next step's grid be scheduled, then waits
-// until the previous grid has completed and its writes are visible, before it
-// touches global memory.
-template <typename T, int Q, int MINB, bool RA = false, bool PDL = false>
-__global__ void __launch_bounds__(256, MINB) k_lbm_step_records(LbmArgs<T> a) {
+// Node layout, G lanes per node: each stencil column costs one index load, (q-1)/2
+// coalesced 8-byte weight loads and lbm_rec_len(q) / 4 16-byte loads of the neighbour's
+// record (FP32 D3Q19: 5, against 9 pair gathers on the pairs layout).  Lane g of a
+// node's group takes the columns g, g + G, ..., the partial sums meet in shuffles and the
+// group's first lane writes.  With G = 1 the same arithmetic, in the same order, as
+// k_lbm_step.  `first`: the warp's first node, a multiple of 32 / G.
+template <typename T, int Q, int G, bool RA, bool PF, int UNR>
+__device__ __forceinline__ void step_records(const LbmArgs<T> &a, int64_t first) {
     using V = typename Vec2<T>::type;
     using W = Vec16<T>;
     using V16 = typename W::type;
     constexpr int NP = (Q - 1) / 2;
     constexpr int RL = lbm_rec_len(Q);
     constexpr int NV = RL / W::n;
-    if constexpr (PDL) {
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-    }
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
+    const int lane = threadIdx.x & 31, g = lane % G;
+    const int64_t i = first + lane / G;
+    const bool live = i < a.n;
+    if (G == 1 && !live) return;
     const int64_t s = i >> 5;
-    const int lane = (int)(i & 31);
     const int n_l = a.n_l;
-    const int32_t *__restrict__ ip = a.idx + ((s * n_l) << 5) + lane;
-    const V *__restrict__ wp = reinterpret_cast<const V *>(a.w) + ((s * NP * (int64_t)n_l) << 5) + lane;
+    const int32_t *__restrict__ ip = a.idx + ((s * n_l) << 5) + (i & 31);
+    const V *__restrict__ wp = reinterpret_cast<const V *>(a.w) + ((s * NP * (int64_t)n_l) << 5) + (i & 31);
     const V16 *__restrict__ rec = reinterpret_cast<const V16 *>(a.fin);
     T f[Q];
 #pragma unroll
     for (int k = 0; k < Q; ++k) f[k] = (T)0;
-#pragma unroll 1
-    for (int j = 0; j < n_l; ++j) {  // not unrolled: keeps the register cap without spills
-        const int q = __ldg(ip + (j << 5));
-        T g[RL];
+    if (live) {
+        // UNR columns in flight; PF: the next column's index is asked for while this one is summed
+        int qn = PF && g < n_l ? __ldg(ip + (g << 5)) : 0;
+#pragma unroll UNR
+        for (int j = g; j < n_l; j += G) {
+            int q;
+            if constexpr (PF) {
+                q = qn;
+                if (j + G < n_l) qn = __ldg(ip + ((j + G) << 5));
+            } else {
+                q = __ldg(ip + (j << 5));
+            }
+            T v[RL];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) W::get(__ldg(rec + (int64_t)q * NV + v), g + v * W::n);
+            for (int t = 0; t < NV; ++t) W::get(__ldg(rec + (int64_t)q * NV + t), v + t * W::n);
 #pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            const V w2 = __ldcs(wp + ((p * n_l + j) << 5));
-            f[2 * p + 1] += w2.x * g[2 * p + 1];
-            f[2 * p + 2] += w2.y * g[2 * p + 2];
+            for (int p = 0; p < NP; ++p) {
+                const V w2 = __ldcs(wp + ((p * n_l + j) << 5));
+                f[2 * p + 1] += w2.x * v[2 * p + 1];
+                f[2 * p + 2] += w2.y * v[2 * p + 2];
+            }
         }
+    }
+    if constexpr (G > 1) {
+#pragma unroll
+        for (int k = 1; k < Q; ++k)
+#pragma unroll
+            for (int off = G >> 1; off > 0; off >>= 1) f[k] += __shfl_xor_sync(0xffffffffu, f[k], off);
+        if (!live || g) return;
     }
     f[0] = a.fin[i * RL];
     const uint32_t m = a.mask[i];
@@ -295,6 +347,31 @@ __global__ void __launch_bounds__(256, MINB) k_lbm_step_records(LbmArgs<T> a) {
     V16 *__restrict__ out = reinterpret_cast<V16 *>(a.fout) + i * NV;
 #pragma unroll
     for (int v = 0; v < NV; ++v) out[v] = W::make(o + v * W::n);
+}
+
+// The step on the node layout, G lanes per node.  MINB: blocks of 256 threads the compiler
+// must fit on one SM, i.e. a register cap.  PDL: launched as a programmatic dependent of the
+// previous kernel in the stream; every block first lets the next step's grid be scheduled,
+// then waits until the previous grid has completed and its writes are visible, before it
+// touches global memory.
+//
+// FP32 is bound by HBM (4 q N_L bytes of weights per node).  Two columns in flight per
+// thread and the next index ahead of them, at 128 registers and 16 warps per SM (MINB 2),
+// beat one column at 64 registers and 32 warps: the bytes in flight are the same, but a
+// wave holds half the nodes and a thread waits half as often.  Measured (us per step, D3Q19,
+// N_L = 30; in brackets one column at 64 registers, and the time of the bytes at the copy
+// bandwidth): 71k nodes 27.5 (32.1, 25.5), 152k 54.9 (57.4, 54.5), 172k 67.1 (94.4, its 672
+// blocks left a nearly empty second wave; 61.6), 261k 102.5 (113, 93.5).
+// FP64 is bound by its pipe (2 lanes per clock and SM): 172k nodes 262 us, 216 for the
+// products alone; the pairs schedule, whose moments every pair repeats, 496.
+template <typename T, int Q, int MINB, int G, bool RA, bool PDL, bool PF, int UNR>
+__global__ void __launch_bounds__(256, MINB) k_lbm_step_records(LbmArgs<T> a) {
+    if constexpr (PDL) {
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    step_records<T, Q, G, RA, PF, UNR>(a, warp * (32 / G));
 }
 
 // Pair-per-warp variant.  A block owns one SELL slice (32 nodes, one per lane)
@@ -357,7 +434,7 @@ __global__ void __launch_bounds__(32 * ((Q - 1) / 2), sizeof(T) == 4 ? 5 : 2) k_
         else if (m & (1u << kb)) ab = ak;
         if (w == 0) f0 = a.fin[i];
     }
-    const T ex = (T)VSet<Q>::e(k, 0), ey = (T)VSet<Q>::e(k, 1), ez = (T)VSet<Q>::e(k, 2);
+    const T ex = (T)c_e<Q>(k, 0), ey = (T)c_e<Q>(k, 1), ez = (T)c_e<Q>(k, 2);
     const T dif = ak - ab;
     part[w][0][lane] = ak + ab + f0;
     part[w][1][lane] = ex * dif;
@@ -499,6 +576,52 @@ cudaError_t lbm_launch_pack_f64(int64_t nc, int q, int n_l, const double *w, dou
     return cudaGetLastError();
 }
 
+template <typename T, int Q, int MINB, int G, bool RA, bool PDL, bool PF, int UNR>
+static cudaError_t launch_records_k(const LbmArgs<T> &a, cudaStream_t st, int block) {
+    const unsigned grid = (unsigned)((a.n * G + block - 1) / block);
+    if constexpr (!PDL) {
+        k_lbm_step_records<T, Q, MINB, G, RA, false, PF, UNR><<<grid, block, 0, st>>>(a);
+        return cudaGetLastError();
+    } else {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(block);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, k_lbm_step_records<T, Q, MINB, G, RA, true, PF, UNR>, a);
+    }
+}
+
+// The node-layout schedules by size.  Cells that leave the chip idle at one lane per node get
+// as many lanes as keep the threads per SM below a limit: FP32 280 (21k nodes: 2 lanes 13.0 us
+// per step, 4 lanes 18.2, 1 lane 15.6; 6k: 4 lanes 7.2, 8 lanes 8.1), FP64 160, because the
+// lanes of a node repeat its collision on the pipe that is the bound (21k: 1 lane 49.4, 2
+// lanes 62; 6k: 4 lanes 29.9, 1 lane 36.0).  block = 0: 64 threads while the grid is small
+// (finer pieces spread more evenly), else 256; FP64 64.  FP64 cells past 320 nodes per SM have
+// the warps to hide the latency and run one column at a time in 128 registers (121k: 191 us
+// against 199).
+template <typename T, int Q, bool RA, bool PDL>
+static cudaError_t launch_records(const LbmArgs<T> &a, cudaStream_t st, int block) {
+    constexpr bool D = sizeof(T) == 8;
+    constexpr int MB = D ? 1 : 2;
+    int lanes = 1;
+    while (lanes < 8 && a.n * lanes * 2 <= (int64_t)a.sms * (D ? 160 : 280)) lanes *= 2;
+    if (block == 0) block = D || a.n * lanes < (int64_t)a.sms * 320 ? 64 : 256;
+    if constexpr (D) {
+        if (a.n > (int64_t)a.sms * 320) return launch_records_k<T, Q, 2, 1, RA, PDL, false, 1>(a, st, block);
+    }
+    switch (lanes) {
+    case 1: return launch_records_k<T, Q, MB, 1, RA, PDL, true, 2>(a, st, block);
+    case 2: return launch_records_k<T, Q, MB, 2, RA, false, true, 2>(a, st, block);
+    case 4: return launch_records_k<T, Q, MB, 4, RA, false, true, 2>(a, st, block);
+    default: return launch_records_k<T, Q, MB, 8, RA, false, true, 2>(a, st, block);
+    }
+}
+
 template <typename T, int Q, bool RA>
 static cudaError_t launch_step_q(const LbmArgs<T> &a, cudaStream_t st, int code) {
     constexpr int NP = (Q - 1) / 2;
@@ -510,33 +633,16 @@ static cudaError_t launch_step_q(const LbmArgs<T> &a, cudaStream_t st, int code)
     case LBM_PAIR_PER_WARP_U3: k_lbm_step_pairs<T, Q, 3, RA><<<slices, 32 * NP, 0, st>>>(a); break;
     case LBM_PAIR_PER_WARP_U6: k_lbm_step_pairs<T, Q, 6, RA><<<slices, 32 * NP, 0, st>>>(a); break;
     case LBM_PAIR_PER_WARP_U2: k_lbm_step_pairs<T, Q, 2, RA><<<slices, 32 * NP, 0, st>>>(a); break;
-    // register caps: FP32 64 / 48 (4 / 5 blocks per SM); FP64 128 / 80 (2 / 3 blocks)
-    case LBM_RECORD_PER_THREAD:
-        k_lbm_step_records<T, Q, sizeof(T) == 4 ? 4 : 2, RA><<<(unsigned)((a.n + 255) / 256), 256, 0, st>>>(a);
-        break;
-    case LBM_RECORD_PER_THREAD_OCC:
-        k_lbm_step_records<T, Q, sizeof(T) == 4 ? 5 : 3, RA><<<(unsigned)((a.n + 255) / 256), 256, 0, st>>>(a);
-        break;
-    case LBM_RECORD_PER_THREAD_128:
-        k_lbm_step_records<T, Q, sizeof(T) == 4 ? 4 : 2, RA><<<(unsigned)((a.n + 127) / 128), 128, 0, st>>>(a);
-        break;
-    case LBM_RECORD_PER_THREAD_64:
-        k_lbm_step_records<T, Q, sizeof(T) == 4 ? 4 : 2, RA><<<(unsigned)((a.n + 63) / 64), 64, 0, st>>>(a);
-        break;
-    case LBM_RECORD_PER_THREAD_PDL: {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)((a.n + 255) / 256));
-        cfg.blockDim = dim3(256);
-        cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_lbm_step_records<T, Q, sizeof(T) == 4 ? 4 : 2, RA, true>, a);
-        if (e != cudaSuccess) return e;
-        break;
-    }
+    case LBM_RECORD_PER_THREAD: return launch_records<T, Q, RA, false>(a, st, 256);
+    case LBM_RECORD_PER_THREAD_128: return launch_records<T, Q, RA, false>(a, st, 128);
+    case LBM_RECORD_PER_THREAD_64: return launch_records<T, Q, RA, false>(a, st, 64);
+    // one column at a time, registers capped for more warps: FP32 48 (5 blocks), FP64 80 (3 blocks)
+    case LBM_RECORD_PER_THREAD_OCC: return launch_records_k<T, Q, sizeof(T) == 4 ? 5 : 3, 1, RA, false, false, 1>(a, st, 256);
+    // Launched programmatically once the grid fills the chip: the steps of an eager run are 2 us
+    // shorter (71k nodes 27.5 against 29.3, 152k 53.8 against 55.8; no difference inside a graph).
+    // The early blocks of the next step crowd a smaller grid (41k nodes: 28.1 against 18.7).
+    case LBM_RECORD_PER_THREAD_PDL:
+        return a.n >= (int64_t)a.sms * 448 ? launch_records<T, Q, RA, true>(a, st, 0) : launch_records<T, Q, RA, false>(a, st, 0);
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

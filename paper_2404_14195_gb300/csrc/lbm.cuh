@@ -25,6 +25,7 @@ struct LbmArgs {
     // refined FP32 (RBF_FP32R): the residual r added to every post-collision
     // population (same layout as fout), else null; FP32 only
     const T *radd = nullptr;
+    int sms = 1;           // SMs of the device (split of the node-layout schedules)
 };
 
 const int *host_velocity_set(int q);
@@ -33,16 +34,15 @@ double host_lattice_weight(int q, int k);
 // schedules of the fused step (same arithmetic, different thread mapping):
 // on the pairs layout, node per thread with 256 / 128 threads per block and
 // pair per warp with the stencil loop unrolled 5 / 3 / 6 / 2 deep; on the node
-// layout, node per thread with 256 threads, registers as needed or capped for
-// five blocks per SM
+// layout, one to eight lanes per node by the size of the cell, in blocks of 256 (6),
+// 128 (8) and 64 (9) threads or by the size of the grid (10), 7 one node per thread with
+// registers capped for more warps
 enum {
     LBM_NODE_PER_THREAD = 0, LBM_PAIR_PER_WARP = 1, LBM_NODE_PER_THREAD_128 = 2,
     LBM_PAIR_PER_WARP_U3 = 3, LBM_PAIR_PER_WARP_U6 = 4, LBM_PAIR_PER_WARP_U2 = 5,
     LBM_RECORD_PER_THREAD = 6, LBM_RECORD_PER_THREAD_OCC = 7,
-    // node layout, node per thread, 64-register kernel in blocks of 128 / 64 threads (finer
-    // blocks spread the nodes more evenly over the SMs in a one-wave launch)
     LBM_RECORD_PER_THREAD_128 = 8, LBM_RECORD_PER_THREAD_64 = 9,
-    // as 6, launched as a programmatic dependent launch: the next step's blocks are
+    // grids that fill the chip are launched programmatically: the next step's blocks are
     // scheduled while this step drains and wait on the hardware grid dependency
     LBM_RECORD_PER_THREAD_PDL = 10, LBM_N_SCHEDULES = 11
 };
