@@ -51,7 +51,7 @@ __host__ __device__ constexpr int64_t b_off_c(int l) { return w_off_c(l) + (int6
 __device__ __forceinline__ int cmo(int r, int k, int K) { return (((r >> 3) * (K >> 3) + (k >> 3)) << 6) + ((r & 7) << 3) + (k & 7); }
 
 // ---- tcgen05 GEMM -------------------------------------------------------------------
-enum { EP_F32 = 0, EP_FWD = 1, EP_OUT = 2, EP_BWD = 3, EP_PRED = 4 };
+enum { EP_F32 = 0, EP_FWD = 1, EP_OUT = 2, EP_BWD = 3 };
 
 struct GemmArgs {
     const bf16 *A;
@@ -60,7 +60,7 @@ struct GemmArgs {
     int ldb;
     int M, N, K;          // M multiple of 128; N in {16, 32, 64, 128}; K multiple of 16, split by gridDim.y
     // epilogue operands
-    float *out32;         // EP_F32: partials [split][M][N]; EP_PRED: [M][4]
+    float *out32;         // EP_F32: partials [split][M][N]
     const float *bias;    // N
     bf16 *H, *Ht, *G;     // EP_FWD / EP_OUT / EP_BWD outputs (row-major [M][N], transposed [N][ldt], G [M][N])
     int ldt;
@@ -187,10 +187,6 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
             float *o = g.out32 + ((int64_t)kid * g.M + m) * N + c0;
 #pragma unroll
             for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4 *>(o + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-        } else if (EP == EP_PRED) {
-            if (c0 == 0 && valid)
-#pragma unroll
-                for (int i = 0; i < N_OUT; ++i) g.out32[(int64_t)m * N_OUT + i] = v[i] + g.bias[i];
         } else {
             __align__(16) bf16 hv[16];
             __align__(16) bf16 gv[16];
@@ -259,7 +255,6 @@ cudaError_t launch_gemm(int ep, const GemmArgs &g, int ksplit, cudaStream_t st) 
     case EP_FWD: k_gemm<EP_FWD><<<grid, 128, GEMM_SMEM, st>>>(g); break;
     case EP_OUT: k_gemm<EP_OUT><<<grid, 128, GEMM_SMEM, st>>>(g); break;
     case EP_BWD: k_gemm<EP_BWD><<<grid, 128, GEMM_SMEM, st>>>(g); break;
-    case EP_PRED: k_gemm<EP_PRED><<<grid, 128, GEMM_SMEM, st>>>(g); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -267,7 +262,7 @@ cudaError_t launch_gemm(int ep, const GemmArgs &g, int ksplit, cudaStream_t st) 
 
 cudaError_t gemm_set_smem() {
     cudaError_t e = cudaSuccess;
-    for (auto f : {k_gemm<EP_F32>, k_gemm<EP_FWD>, k_gemm<EP_OUT>, k_gemm<EP_BWD>, k_gemm<EP_PRED>}) {
+    for (auto f : {k_gemm<EP_F32>, k_gemm<EP_FWD>, k_gemm<EP_OUT>, k_gemm<EP_BWD>}) {
         e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM);
         if (e != cudaSuccess) return e;
     }
@@ -462,6 +457,7 @@ struct FusedArgs {
     bf16 *dY;                    // B x 16 in the chunked layout of chunk_off
     float *loss, *grad;
     float gscale;
+    float *pred;                 // prediction only: outputs [n][4]
     int32_t *err;
 };
 
@@ -532,13 +528,52 @@ __device__ __forceinline__ float warp_colsum16(const float *v, int lane, int &co
 // 8 BF16 values as one 16-byte word
 __device__ __forceinline__ uint4 pack8(const bf16 *v) { return *reinterpret_cast<const uint4 *>(v); }
 
+constexpr int wave(int j, int a) {  // c_waves as compile-time constants in unrolled code
+    constexpr int t[16][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1},  {1, 1, 0},   {1, -1, 0}, {1, 0, 1},
+                              {1, 0, -1}, {0, 1, 1},  {0, 1, -1}, {1, 1, 1},   {1, 1, -1}, {1, -1, 1},
+                              {1, -1, -1}, {2, 0, 0}, {0, 2, 0},  {0, 0, 2}};
+    return t[j][a];
+}
+// whether an error of up to 1e-6 in v could change its rounding to BF16
+__device__ __forceinline__ bool bf16_unsure(float v) {
+    const float mid = __uint_as_float((__float_as_uint(v) & 0xffff0000u) | 0x8000u);
+    return !(fabsf(v - mid) > 1e-6f);
+}
+// BF16 sine and cosine of 2 pi n_j . x as one word, the same bits as the FP64 values rounded (k_features):
+// the phase is reduced in FP64, the functions are evaluated in FP32 on its leading part with
+// a first-order correction by the rest (error below 3e-7), and the few values that lie within
+// 1e-6 of a rounding boundary are evaluated in FP64.  FP64 sincospi for all of them was most
+// of the feature kernel's time.
+__device__ __forceinline__ uint32_t bf16_pair(bf16 lo, bf16 hi) {
+    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+}
+__device__ __forceinline__ uint32_t wave_feature(int j, double x, double y, double z) {
+    const double ph = wave(j, 0) * x + wave(j, 1) * y + wave(j, 2) * z;
+    const double fr = ph - rint(ph);
+    const float hi = (float)fr, lo = 6.283185307f * (float)(fr - (double)hi);
+    float s0, c0;
+    sincospif(2.0f * hi, &s0, &c0);
+    const float s = fmaf(c0, lo, s0), c = fmaf(-s0, lo, c0);
+    if (bf16_unsure(s) || bf16_unsure(c)) {
+        double sd, cd;
+        sincospi(2.0 * ph, &sd, &cd);
+        return bf16_pair(__double2bfloat16(sd), __double2bfloat16(cd));
+    }
+    return bf16_pair(__float2bfloat16(s), __float2bfloat16(c));
+}
+
 // Both kernels run 256 threads per tile: thread t serves row t % 128 of the tile (TMEM
 // lane t % 128, reachable by warps w and w + 4) and half h = t / 128 of each layer's
 // columns, so two warps per scheduler share the epilogue math.  The forward kernel
 // runs NG such tile groups per CTA on the shared resident weights, each with its own
 // activation tile, TMEM columns, mbarrier and named barrier: while one group's
 // epilogue runs, the other's MMAs keep the tensor pipe busy.
-template <int NG>
+//
+// PRED: prediction of the f.n points themselves (row r = point r), features as k_features
+// rounds them; only the outputs leave the chip, f.pred [n][4].  60,001 points: one
+// launch of 65 us in place of 4 chunks of a feature kernel and five GEMMs (24 + 5 x 20 us each),
+// a call 867 -> 177 us with its copies.
+template <int NG, bool PRED = false>
 __global__ void __launch_bounds__(256 * NG, 1) k_mlp_fwd(FusedArgs f) {
     extern __shared__ __align__(1024) uint8_t smem[];
     bf16 *sW[N_LAYERS];
@@ -580,51 +615,54 @@ __global__ void __launch_bounds__(256 * NG, 1) k_mlp_fwd(FusedArgs f) {
     bool ok = tc::mbar_wait(wbar, 0, WAIT_NS);
     uint32_t phase = 0;
     float lsum = 0.0f;
-    for (int tile = blockIdx.x * NG + grp; ok && tile < (f.B >> 7); tile += gridDim.x * NG) {
+    const int tiles = PRED ? (int)((f.n + 127) >> 7) : f.B >> 7;
+    for (int tile = blockIdx.x * NG + grp; ok && tile < tiles; tile += gridDim.x * NG) {
         const int64_t r = (int64_t)tile * 128 + row;
         int64_t s;
-        if (f.idx) s = f.idx[r];
+        if (PRED) s = r < f.n ? r : f.n - 1;
+        else if (f.idx) s = f.idx[r];
         else {
             const uint64_t c = f.seed * (1ull << 32) + (uint64_t)(*f.step_dev) * (uint64_t)f.B + (uint64_t)r;
             s = (int64_t)(splitmix64(c) % (uint64_t)f.n);
         }
         {   // features of sample s (half h: wave vectors 8h .. 8h + 7; half 0 also r and
-            // phi_sdf): the sines and cosines of k_features, evaluated in FP32 on the
+            // phi_sdf): training evaluates the sines and cosines of k_features in FP32 on the
             // coordinates reduced to [0, 1) (periodic, so exact up to float rounding,
             // ~1e-7, far below the BF16 resolution the features are stored at)
             const double x = f.xyz[3 * s], y = f.xyz[3 * s + 1], z = f.xyz[3 * s + 2];
             const float xf = (float)(x - floor(x)), yf = (float)(y - floor(y)), zf = (float)(z - floor(z));
-            __align__(16) bf16 part[32];
+            // columns 16 half .. + 15 (sines and cosines of wave vectors 8 half ..) as eight two-value
+            // words, then columns 32 + 16 half .. (half 0: r, phi_sdf, zeros; half 1: zeros)
+            uint32_t wv[8];
 #pragma unroll
             for (int jj = 0; jj < 8; ++jj) {
-                const int j = 8 * half + jj;
-                float sn, cs;
-                sincospif(2.0f * ((float)c_waves[j][0] * xf + (float)c_waves[j][1] * yf + (float)c_waves[j][2] * zf), &sn,
-                          &cs);
-                part[2 * jj] = __float2bfloat16(sn);
-                part[2 * jj + 1] = __float2bfloat16(cs);
+                if constexpr (PRED) {
+                    wv[jj] = half ? wave_feature(8 + jj, x, y, z) : wave_feature(jj, x, y, z);
+                } else {
+                    const int j = 8 * half + jj;
+                    float sn, cs;
+                    sincospif(2.0f * ((float)c_waves[j][0] * xf + (float)c_waves[j][1] * yf + (float)c_waves[j][2] * zf), &sn,
+                              &cs);
+                    wv[jj] = bf16_pair(__float2bfloat16(sn), __float2bfloat16(cs));
+                }
             }
-#pragma unroll
-            for (int j = 16; j < 32; ++j) part[j] = __float2bfloat16(0.0f);
-            if (half == 0) {
-                part[16] = __float2bfloat16(f.rad[s]);  // columns 32, 33 of the row
-                part[17] = __float2bfloat16(f.sdf[s]);
-            }
-            // half 0 owns columns 0..15 and 32..47 (r, phi_sdf, zeros), half 1 columns
-            // 16..31 and 48..63 (zeros): each written as two 16-column pieces
+            const uint32_t geo = half ? 0u : bf16_pair(__float2bfloat16(f.rad[s]), __float2bfloat16(f.sdf[s]));
             const int cA = 16 * half, cB = 32 + 16 * half;
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                const uint4 wA = pack8(part + 8 * k), wB = pack8(part + 16 + 8 * k);
+                const uint4 wA = make_uint4(wv[4 * k], wv[4 * k + 1], wv[4 * k + 2], wv[4 * k + 3]);
+                const uint4 wB = make_uint4(k ? 0u : geo, 0u, 0u, 0u);
                 *reinterpret_cast<uint4 *>(act + cmo(row, cA + 8 * k, N_IN)) = wA;
                 *reinterpret_cast<uint4 *>(act + cmo(row, cB + 8 * k, N_IN)) = wB;
-                *reinterpret_cast<uint4 *>(f.X + chunk_off<N_IN / 8>(r, (cA >> 3) + k)) = wA;
-                *reinterpret_cast<uint4 *>(f.X + chunk_off<N_IN / 8>(r, (cB >> 3) + k)) = wB;
+                if constexpr (!PRED) {
+                    *reinterpret_cast<uint4 *>(f.X + chunk_off<N_IN / 8>(r, (cA >> 3) + k)) = wA;
+                    *reinterpret_cast<uint4 *>(f.X + chunk_off<N_IN / 8>(r, (cB >> 3) + k)) = wB;
+                }
             }
         }
         float tg[N_OUT];
 #pragma unroll
-        for (int c = 0; c < N_OUT; ++c) tg[c] = half ? 0.0f : f.tgt[s * N_OUT + c];
+        for (int c = 0; c < N_OUT; ++c) tg[c] = half || PRED ? 0.0f : f.tgt[s * N_OUT + c];
         for (int l = 0; l < N_LAYERS && ok; ++l) {
             const int fi = fan_in(l), fo = fan_out(l);
             if (NG == 1) smem_to_mma_sync();
@@ -647,41 +685,47 @@ __global__ void __launch_bounds__(256 * NG, 1) k_mlp_fwd(FusedArgs f) {
                         const float4 q = reinterpret_cast<const float4 *>(bias + c0)[k];
                         v[4 * k] += q.x; v[4 * k + 1] += q.y; v[4 * k + 2] += q.z; v[4 * k + 3] += q.w;
                     }
-                    __align__(16) __nv_bfloat162 hv2[8];
-                    __align__(16) __nv_bfloat162 gv2[8];
+                    uint32_t hw[8], gw[8];  // BF16 pairs, as words
 #pragma unroll
                     for (int i = 0; i < 16; i += 2) {  // pairs: one two-value conversion each
                         float h0, g0, h1, g1;
                         gelu_both(v[i], h0, g0);
                         gelu_both(v[i + 1], h1, g1);
-                        hv2[i >> 1] = __floats2bfloat162_rn(h0, h1);
-                        gv2[i >> 1] = __floats2bfloat162_rn(g0, g1);
+                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(h0, h1), g2 = __floats2bfloat162_rn(g0, g1);
+                        hw[i >> 1] = bf16_pair(h2.x, h2.y);
+                        gw[i >> 1] = bf16_pair(g2.x, g2.y);
                     }
-                    const bf16 *hv = reinterpret_cast<const bf16 *>(hv2), *gv = reinterpret_cast<const bf16 *>(gv2);
-                    *reinterpret_cast<uint4 *>(act + cmo(row, c0, N_H)) = pack8(hv);
-                    *reinterpret_cast<uint4 *>(act + cmo(row, c0 + 8, N_H)) = pack8(hv + 8);
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
-                        *reinterpret_cast<uint4 *>(f.H[l] + hg_off(r, (c0 >> 3) + k)) = pack8(hv + 8 * k);
-                        *reinterpret_cast<uint4 *>(f.G[l] + hg_off(r, (c0 >> 3) + k)) = pack8(gv + 8 * k);
+                        const uint4 h4 = make_uint4(hw[4 * k], hw[4 * k + 1], hw[4 * k + 2], hw[4 * k + 3]);
+                        *reinterpret_cast<uint4 *>(act + cmo(row, c0 + 8 * k, N_H)) = h4;
+                        if constexpr (!PRED) {
+                            *reinterpret_cast<uint4 *>(f.H[l] + hg_off(r, (c0 >> 3) + k)) = h4;
+                            *reinterpret_cast<uint4 *>(f.G[l] + hg_off(r, (c0 >> 3) + k)) =
+                                make_uint4(gw[4 * k], gw[4 * k + 1], gw[4 * k + 2], gw[4 * k + 3]);
+                        }
                     }
                 }
             } else if (half == 0) {
                 float v[16];
                 tc::tmem_ld16(tmem + tlane, v);
-                __align__(16) bf16 dv[16];
+                if constexpr (PRED) {
+                    if (r < f.n)
+                        reinterpret_cast<float4 *>(f.pred)[r] =
+                            make_float4(v[0] + bias[0], v[1] + bias[1], v[2] + bias[2], v[3] + bias[3]);
+                } else {
+                    float dy[N_OUT];
 #pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    float dy = 0.0f;
-                    if (c < N_OUT) {
+                    for (int c = 0; c < N_OUT; ++c) {
                         const float e = v[c] + bias[c] - tg[c];
                         lsum += e * e;
-                        dy = f.gscale * e;
+                        dy[c] = f.gscale * e;
                     }
-                    dv[c] = __float2bfloat16(dy);
+                    *reinterpret_cast<uint4 *>(f.dY + chunk_off<N_OUT_PAD / 8>(r, 0)) =
+                        make_uint4(bf16_pair(__float2bfloat16(dy[0]), __float2bfloat16(dy[1])),
+                                   bf16_pair(__float2bfloat16(dy[2]), __float2bfloat16(dy[3])), 0u, 0u);
+                    *reinterpret_cast<uint4 *>(f.dY + chunk_off<N_OUT_PAD / 8>(r, 1)) = make_uint4(0u, 0u, 0u, 0u);
                 }
-                *reinterpret_cast<uint4 *>(f.dY + chunk_off<N_OUT_PAD / 8>(r, 0)) = pack8(dv);
-                *reinterpret_cast<uint4 *>(f.dY + chunk_off<N_OUT_PAD / 8>(r, 1)) = pack8(dv + 8);
             }
             tc::fence_before_sync();
         }
@@ -690,8 +734,10 @@ __global__ void __launch_bounds__(256 * NG, 1) k_mlp_fwd(FusedArgs f) {
         if (gt == 0) atomicExch(f.err, 1);
         tc::mbar_wait(mbar, phase, WAIT_NS);
     }
-    for (int off = 16; off > 0; off >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
-    if (lane == 0 && lsum != 0.0f) atomicAdd(f.loss, lsum);
+    if constexpr (!PRED) {
+        for (int off = 16; off > 0; off >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
+        if (lane == 0 && lsum != 0.0f) atomicAdd(f.loss, lsum);
+    }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(*slot, 128 * NG);
@@ -942,6 +988,8 @@ __global__ void __launch_bounds__(256, 1) k_mlp_bwd(FusedArgs f) {
 cudaError_t fused_set_smem() {
     cudaError_t e = cudaFuncSetAttribute(k_mlp_fwd<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fw_smem(1));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_fwd<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fw_smem(2));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_fwd<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fw_smem(1));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_fwd<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fw_smem(2));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FB_SMEM);
     return e;
 }
@@ -968,7 +1016,8 @@ struct rbf_mlp {
     // workspace for batch B
     int B = 0;
     DevArr<bf16> X, Xt, H[4], Ht[4], G[4], dY, dYt, dZ[4], dZt[4];
-    DevArr<float> T, part, loss, pred;
+    DevArr<float> T, part, loss;
+    DevArr<char> pws;  // predictions: points and outputs of the largest call so far
     DevArr<int64_t> idx;
     DevArr<int32_t> errflag;
     cudaGraphExec_t gexec = nullptr;
@@ -1033,7 +1082,6 @@ int ensure_workspace(rbf_mlp *mm, int B) {
     MCK(mm->dY.alloc((size_t)B * N_OUT_PAD));
     MCK(mm->dYt.alloc((size_t)B * N_OUT_PAD));
     MCK(mm->T.alloc((size_t)B * N_OUT));
-    MCK(mm->pred.alloc((size_t)B * N_OUT));
     MCK(mm->idx.alloc((size_t)B));
     MCK(mm->part.alloc((size_t)(B / 128) * N_H * N_H));
     mm->B = B;
@@ -1047,9 +1095,9 @@ GemmArgs gemm_args(const bf16 *A, int lda, const bf16 *Bm, int ldb, int M, int N
     return g;
 }
 
-// forward of the B rows in X; train: keep activations, transposes and GELU' and
-// the loss gradient (targets T); otherwise write predictions to pred
-cudaError_t enqueue_forward(rbf_mlp *mm, int B, int nvalid, bool train) {
+// training forward of the B rows in X, one GEMM per layer: keeps activations, transposes,
+// GELU' and the loss gradient (targets T)
+cudaError_t enqueue_forward(rbf_mlp *mm, int B) {
     cudaError_t e;
     const bf16 *in = mm->X.p;
     int fin = N_IN;
@@ -1057,10 +1105,9 @@ cudaError_t enqueue_forward(rbf_mlp *mm, int B, int nvalid, bool train) {
         GemmArgs g = gemm_args(in, fin, mm->W[l].p, fan_in(l), B, N_H, fin, mm->errflag.p);
         g.bias = mm->theta.p + b_off(l);
         g.H = mm->H[l].p;
-        g.Ht = train ? mm->Ht[l].p : nullptr;
-        g.G = train ? mm->G[l].p : nullptr;
+        g.Ht = mm->Ht[l].p;
+        g.G = mm->G[l].p;
         g.ldt = B;
-        g.nvalid = nvalid;
         if ((e = launch_gemm(EP_FWD, g, 1, mm->st)) != cudaSuccess) return e;
         ++mm->launches;
         in = mm->H[l].p;
@@ -1068,23 +1115,44 @@ cudaError_t enqueue_forward(rbf_mlp *mm, int B, int nvalid, bool train) {
     }
     GemmArgs g = gemm_args(in, N_H, mm->W[4].p, N_H, B, N_OUT_PAD, N_H, mm->errflag.p);
     g.bias = mm->theta.p + b_off(4);
-    g.nvalid = nvalid;
-    if (train) {
-        g.T = mm->T.p;
-        g.H = mm->dY.p;
-        g.Ht = mm->dYt.p;
-        g.ldt = B;
-        g.loss = mm->loss.p;
-        g.db = mm->grad.p + b_off(4);
-        g.gscale = 2.0f / ((float)nvalid * N_OUT);
-        e = launch_gemm(EP_OUT, g, 1, mm->st);
-    } else {
-        g.out32 = mm->pred.p;
-        e = launch_gemm(EP_PRED, g, 1, mm->st);
-    }
+    g.T = mm->T.p;
+    g.H = mm->dY.p;
+    g.Ht = mm->dYt.p;
+    g.ldt = B;
+    g.loss = mm->loss.p;
+    g.db = mm->grad.p + b_off(4);
+    g.gscale = 2.0f / ((float)B * N_OUT);
+    e = launch_gemm(EP_OUT, g, 1, mm->st);
     ++mm->launches;
     return e;
 }
+
+// outputs [n][4] of the n points in one launch of the fused forward
+cudaError_t enqueue_predict(rbf_mlp *mm, int64_t n, const double *xyz, const float *rad, const float *sdf, float *out) {
+    FusedArgs f;
+    std::memset(&f, 0, sizeof(f));
+    f.n = n; f.xyz = xyz; f.rad = rad; f.sdf = sdf; f.pred = out;
+    for (int l = 0; l < N_LAYERS; ++l) f.Wc[l] = mm->Wc[l].p;
+    f.theta = mm->theta.p;
+    f.err = mm->errflag.p;
+    const int64_t tiles = (n + 127) / 128, nsm = std::max(mm->nsm, 1);
+    if (tiles > nsm) k_mlp_fwd<2, true><<<(unsigned)std::min<int64_t>((tiles + 1) / 2, nsm), 512, fw_smem(2), mm->st>>>(f);
+    else k_mlp_fwd<1, true><<<(unsigned)tiles, 256, fw_smem(1), mm->st>>>(f);
+    ++mm->launches;
+    return cudaGetLastError();
+}
+
+// byte offsets of a prediction's arrays in pws: points, radii, wall distances, outputs
+struct PredLayout {
+    size_t rad, sdf, out, total;
+    explicit PredLayout(size_t n) {
+        auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+        rad = up(3 * n * sizeof(double));
+        sdf = rad + up(n * sizeof(float));
+        out = sdf + up(n * sizeof(float));
+        total = out + up(N_OUT * n * sizeof(float));
+    }
+};
 
 // backward: gradient of the mean squared error into mm->grad (packed layout)
 cudaError_t enqueue_backward(rbf_mlp *mm, int B) {
@@ -1169,7 +1237,7 @@ cudaError_t enqueue_train_step(rbf_mlp *mm, int B, uint64_t seed, float lr, cons
                                                         explicit_idx, seed, mm->counters.p + 1, mm->X.p, mm->Xt.p, B,
                                                         mm->T.p);
         ++mm->launches;
-        if ((e = enqueue_forward(mm, B, B, true)) != cudaSuccess) return e;
+        if ((e = enqueue_forward(mm, B)) != cudaSuccess) return e;
         if ((e = enqueue_backward(mm, B)) != cudaSuccess) return e;
     }
     if (update) {
@@ -1344,28 +1412,14 @@ int rbf_mlp_train(rbf_mlp *mm, int steps, int batch, double lr, uint64_t seed, f
 int rbf_mlp_predict(rbf_mlp *mm, int64_t n, const double *xyz, const float *radius, const float *sdf, float *out) {
     if (!mm || n < 1 || !xyz || !radius || !sdf || !out) return RBF_EINVAL;
     MDevGuard dg(mm->device);
-    const int B = 16384;
-    int rc = ensure_workspace(mm, std::max(mm->B, B));
-    if (rc) return rc;
-    const int Bw = mm->B;
-    DevArr<double> px;
-    DevArr<float> pr, ps;
-    MCK(px.alloc(3 * n)); MCK(pr.alloc(n)); MCK(ps.alloc(n));
-    MCK(cudaMemcpyAsync(px.p, xyz, 3 * n * sizeof(double), cudaMemcpyHostToDevice, mm->st));
-    MCK(cudaMemcpyAsync(pr.p, radius, n * sizeof(float), cudaMemcpyHostToDevice, mm->st));
-    MCK(cudaMemcpyAsync(ps.p, sdf, n * sizeof(float), cudaMemcpyHostToDevice, mm->st));
-    std::vector<int64_t> ids(Bw);
-    for (int64_t s0 = 0; s0 < n; s0 += Bw) {
-        const int cnt = (int)std::min<int64_t>(Bw, n - s0);
-        for (int b = 0; b < Bw; ++b) ids[b] = b < cnt ? s0 + b : s0;
-        MCK(cudaMemcpyAsync(mm->idx.p, ids.data(), Bw * sizeof(int64_t), cudaMemcpyHostToDevice, mm->st));
-        k_features<<<(Bw + 127) / 128, 128, 0, mm->st>>>(Bw, n, px.p, pr.p, ps.p, nullptr, mm->idx.p, 0, mm->counters.p + 1,
-                                                        mm->X.p, nullptr, Bw, nullptr);
-        ++mm->launches;
-        MCK(enqueue_forward(mm, Bw, cnt, false));
-        MCK(cudaMemcpyAsync(out + 4 * s0, mm->pred.p, (size_t)cnt * 4 * sizeof(float), cudaMemcpyDeviceToHost, mm->st));
-        MCK(cudaStreamSynchronize(mm->st));  // ids is reused
-    }
+    const PredLayout pl((size_t)n);
+    if (mm->pws.n < pl.total) MCK(mm->pws.alloc(pl.total));
+    char *w = mm->pws.p;
+    MCK(cudaMemcpyAsync(w, xyz, 3 * n * sizeof(double), cudaMemcpyHostToDevice, mm->st));
+    MCK(cudaMemcpyAsync(w + pl.rad, radius, n * sizeof(float), cudaMemcpyHostToDevice, mm->st));
+    MCK(cudaMemcpyAsync(w + pl.sdf, sdf, n * sizeof(float), cudaMemcpyHostToDevice, mm->st));
+    MCK(enqueue_predict(mm, n, (const double *)w, (const float *)(w + pl.rad), (const float *)(w + pl.sdf), (float *)(w + pl.out)));
+    MCK(cudaMemcpyAsync(out, w + pl.out, N_OUT * n * sizeof(float), cudaMemcpyDeviceToHost, mm->st));
     return check_err(mm);
 }
 
@@ -1378,31 +1432,18 @@ int rbf_mlp_warm_start(rbf_mlp *mm, rbf_ctx *ctx, const double *scale) {
     const int64_t n = ctx->n;
     // order the context's stream after the network's
     MCK(cudaStreamSynchronize(ctx->st));
-    int rc = ensure_workspace(mm, std::max(mm->B, 16384));
-    if (rc) return rc;
-    const int Bw = mm->B;
-    DevArr<float> rad, sdf, predall;
-    MCK(rad.alloc(n)); MCK(sdf.alloc(n)); MCK(predall.alloc(4 * n));
-    k_node_geo<<<(unsigned)((n + 255) / 256), 256, 0, mm->st>>>(n, ctx->xyz.p, ctx->c[0], ctx->c[1], ctx->c[2], ctx->r, rad.p, sdf.p);
+    const PredLayout pl((size_t)n);
+    if (mm->pws.n < pl.total) MCK(mm->pws.alloc(pl.total));
+    float *rad = (float *)(mm->pws.p + pl.rad), *sdf = (float *)(mm->pws.p + pl.sdf), *pred = (float *)(mm->pws.p + pl.out);
+    k_node_geo<<<(unsigned)((n + 255) / 256), 256, 0, mm->st>>>(n, ctx->xyz.p, ctx->c[0], ctx->c[1], ctx->c[2], ctx->r, rad, sdf);
     ++mm->launches;
-    std::vector<int64_t> ids(Bw);
-    for (int64_t s0 = 0; s0 < n; s0 += Bw) {
-        const int cnt = (int)std::min<int64_t>(Bw, n - s0);
-        for (int b = 0; b < Bw; ++b) ids[b] = b < cnt ? s0 + b : s0;
-        MCK(cudaMemcpyAsync(mm->idx.p, ids.data(), Bw * sizeof(int64_t), cudaMemcpyHostToDevice, mm->st));
-        k_features<<<(Bw + 127) / 128, 128, 0, mm->st>>>(Bw, n, ctx->xyz.p, rad.p, sdf.p, nullptr, mm->idx.p, 0,
-                                                        mm->counters.p + 1, mm->X.p, nullptr, Bw, nullptr);
-        ++mm->launches;
-        MCK(enqueue_forward(mm, Bw, cnt, false));
-        MCK(cudaMemcpyAsync(predall.p + 4 * s0, mm->pred.p, (size_t)cnt * 4 * sizeof(float), cudaMemcpyDeviceToDevice, mm->st));
-        MCK(cudaStreamSynchronize(mm->st));
-    }
+    MCK(enqueue_predict(mm, n, ctx->xyz.p, rad, sdf, pred));
     const unsigned gb = (unsigned)((n + 255) / 256);
     const float4 sc = make_float4((float)scale[0], (float)scale[1], (float)scale[2], (float)scale[3]);
     if (ctx->prec != RBF_FP64)
-        k_inject<float><<<gb, 256, 0, mm->st>>>(n, predall.p, ctx->type.p, sc, ctx->a32[0].p, ctx->a32[1].p, ctx->a32[2].p, ctx->a32[3].p);
+        k_inject<float><<<gb, 256, 0, mm->st>>>(n, pred, ctx->type.p, sc, ctx->a32[0].p, ctx->a32[1].p, ctx->a32[2].p, ctx->a32[3].p);
     else
-        k_inject<double><<<gb, 256, 0, mm->st>>>(n, predall.p, ctx->type.p, sc, ctx->a64[0].p, ctx->a64[1].p, ctx->a64[2].p, ctx->a64[3].p);
+        k_inject<double><<<gb, 256, 0, mm->st>>>(n, pred, ctx->type.p, sc, ctx->a64[0].p, ctx->a64[1].p, ctx->a64[2].p, ctx->a64[3].p);
     ++mm->launches;
     if (ctx->prec == RBF_FP32C)
         for (int c = 0; c < 4; ++c) MCK(ctx->l32[c].zero(mm->st));
