@@ -515,26 +515,25 @@ int rbf_build_stencils(rbf_ctx *ctx, int n_l) {
     G = std::max(1, std::min(G, 400));
     ctx->G = G;
     const int64_t ncell = (int64_t)G * G * G;
-    DevArr<int32_t> cell_of, counts, fill, tmp;
+    DevArr<int32_t> cell_of, counts, fill, items, tmp;
     CK(cell_of.alloc(n)); CK(counts.alloc(ncell + 1)); CK(fill.alloc(ncell));
-    CK(ctx->cstart.alloc(ncell + 1)); CK(ctx->citems.alloc(n)); CK(tmp.alloc(scan_tmp_len(ncell + 1)));
+    CK(ctx->cstart.alloc(ncell + 1)); CK(items.alloc(n)); CK(ctx->cpts.alloc(n)); CK(tmp.alloc(scan_tmp_len(ncell + 1)));
     CK(counts.zero(ctx->st)); CK(fill.zero(ctx->st));
     CK(launch_cell_count(n, ctx->xyz.p, G, cell_of.p, counts.p, ctx->st));
     CK(launch_scan_i32(counts.p, ctx->cstart.p, ncell + 1, tmp.p, tmp.n, ctx->st, &ctx->launches));
-    CK(launch_cell_fill(n, cell_of.p, ctx->cstart.p, fill.p, ctx->citems.p, ctx->st));
-    ctx->launches += 2;
+    CK(launch_cell_fill(n, cell_of.p, ctx->cstart.p, fill.p, items.p, ctx->st));
+    CK(launch_cell_points(n, items.p, ctx->xyz.p, ctx->type.p, ctx->cpts.p, ctx->st));
+    ctx->launches += 3;
     CK(ctx->idx.alloc(n * n_l));
     CK(ctx->status.zero(ctx->st));
-    CK(launch_knn(n, nullptr, ctx->iota.p, ctx->xyz.p, ctx->perm.p, ctx->type.p, 0, G, ctx->cstart.p,
-                  ctx->citems.p, n_l, ctx->idx.p, n_l, 0, ctx->status.p, ctx->st));
+    CK(launch_knn(n, nullptr, ctx->iota.p, ctx->xyz.p, ctx->perm.p, 0, G, ctx->cstart.p, ctx->cpts.p, n_l, ctx->idx.p, n_l, 0, ctx->status.p, ctx->st));
     ++ctx->launches;
     CK(ctx->idxb.alloc(ctx->nb * n_l));
     CK(ctx->idxw.alloc(ctx->nb * n_l));
     if (ctx->nb > 0) {
         CK(cudaMemcpy2DAsync(ctx->idxb.p, n_l * sizeof(int32_t), ctx->wall.p, sizeof(int32_t), sizeof(int32_t),
                              ctx->nb, cudaMemcpyDeviceToDevice, ctx->st));
-        CK(launch_knn(ctx->nb, nullptr, ctx->wall.p, ctx->xyz.p, ctx->perm.p, ctx->type.p, 1, G, ctx->cstart.p,
-                      ctx->citems.p, n_l - 1, ctx->idxb.p, n_l, 1, ctx->status.p, ctx->st));
+        CK(launch_knn(ctx->nb, nullptr, ctx->wall.p, ctx->xyz.p, ctx->perm.p, 1, G, ctx->cstart.p, ctx->cpts.p, n_l - 1, ctx->idxb.p, n_l, 1, ctx->status.p, ctx->st));
         k_gather_rows<<<nblk(ctx->nb * n_l), 256, 0, ctx->st>>>(ctx->nb, n_l, ctx->wall.p, ctx->idx.p, ctx->idxw.p);
         ctx->launches += 2;
     }
@@ -1210,8 +1209,7 @@ int ensure_probes(rbf_ctx *ctx, int m_p) {
     CK(pw.alloc(std::max<int64_t>(nfl, 1) * n_l));
     CK(ctx->status.zero(ctx->st));
     if (nfl > 0) {
-        CK(launch_knn(nfl, pxyz.p, nullptr, ctx->xyz.p, ctx->perm.p, ctx->type.p, 0, ctx->G, ctx->cstart.p,
-                      ctx->citems.p, n_l, pidx.p, n_l, 0, ctx->status.p, ctx->st));
+        CK(launch_knn(nfl, pxyz.p, nullptr, ctx->xyz.p, ctx->perm.p, 0, ctx->G, ctx->cstart.p, ctx->cpts.p, n_l, pidx.p, n_l, 0, ctx->status.p, ctx->st));
         OpSpec op{OP_INTERP, {0.0, 0.0, 0.0}};
         DevArr<OpSpec> d_op;
         CK(d_op.alloc(1));

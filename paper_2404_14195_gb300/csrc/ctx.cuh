@@ -57,7 +57,8 @@ struct rbf_ctx {
     double c[3] = {0.5, 0.5, 0.5}, r = 0.0;
     // stencils
     int G = 0, n_l = 0;
-    DevArr<int32_t> cstart, citems, idx, idxb, idxw, idx_sell, idxb_sell;
+    DevArr<float4> cpts;  // cell-sorted points of the neighbour search
+    DevArr<int32_t> cstart, idx, idxb, idxw, idx_sell, idxb_sell;
     // weights
     bool weights_ok = false;
     int solver = -1, q = 0, phs_k = 0, mono_m = 0, n_ops = 0;

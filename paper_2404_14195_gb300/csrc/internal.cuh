@@ -66,12 +66,14 @@ cudaError_t launch_cell_fill(int64_t n, const int32_t *cell_of, const int32_t *s
 cudaError_t launch_flag_compact(int64_t n, const uint8_t *type, uint8_t want, const int32_t *scan,
                                 int32_t *list, cudaStream_t st);
 cudaError_t launch_type_flags(int64_t n, const uint8_t *type, uint8_t want, int32_t *flags, cudaStream_t st);
+// cell-sorted FP32 points of the neighbour search, {x, y, z, node | wall << 31}
+cudaError_t launch_cell_points(int64_t n, const int32_t *items, const double *xyz, const uint8_t *type, float4 *pts,
+                               cudaStream_t st);
 // kNN of nq query points (qxyz, or the nodes qnode[] when qxyz == NULL) among the
 // sorted nodes; results sorted by (d^2, orig index); fluid_only skips wall nodes.
-// out row stride `ld`, first column `col0`.
-cudaError_t launch_knn(int64_t nq, const double *qxyz, const int32_t *qnode, const double *xyz,
-                       const int32_t *perm, const uint8_t *type, int fluid_only, int G,
-                       const int32_t *cell_start, const int32_t *cell_items, int n_l, int32_t *out,
+// n_l <= 64; out row stride `ld`, first column `col0`.
+cudaError_t launch_knn(int64_t nq, const double *qxyz, const int32_t *qnode, const double *xyz, const int32_t *perm,
+                       int fluid_only, int G, const int32_t *cell_start, const float4 *pts, int n_l, int32_t *out,
                        int ld, int col0, int32_t *status, cudaStream_t st);
 
 // weights.cu

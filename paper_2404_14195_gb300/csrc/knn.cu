@@ -5,7 +5,7 @@
 // Nodes are sorted along a 3-D Morton curve (21 bits per axis) so that the nodes
 // of one warp are close in space and the stencil gathers of the step kernels hit
 // the same cache lines.  Neighbour search uses a uniform periodic cell grid and
-// expanding Chebyshev rings; candidates are ranked by (squared distance computed
+// boxes of cells around the query; candidates are ranked by (squared distance computed
 // without FMA, caller's node index), which makes the stencils bitwise
 // reproducible and independent of the internal order.
 #include "internal.cuh"
@@ -264,24 +264,102 @@ cudaError_t launch_flag_compact(int64_t n, const uint8_t *type, uint8_t want, co
     return cudaGetLastError();
 }
 
+// Cell-sorted copies for the neighbour search: FP32 coordinates and the node number, its
+// top bit set for wall nodes
+__global__ void k_cell_points(int64_t n, const int32_t *__restrict__ items, const double *__restrict__ xyz,
+                              const uint8_t *__restrict__ type, float4 *__restrict__ pts) {
+    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const int64_t s = items[e];
+    pts[e] = make_float4((float)xyz[3 * s], (float)xyz[3 * s + 1], (float)xyz[3 * s + 2],
+                         __uint_as_float((uint32_t)s | (type[s] ? 0x80000000u : 0u)));
+}
+
+cudaError_t launch_cell_points(int64_t n, const int32_t *items, const double *xyz, const uint8_t *type, float4 *pts,
+                               cudaStream_t st) {
+    k_cell_points<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, items, xyz, type, pts);
+    return cudaGetLastError();
+}
+
 // ---- k nearest neighbours ---------------------------------------------------
-// One thread per query.  The best n_l candidates are kept sorted in local memory
-// by (d2, orig).  Rings of cells at Chebyshev distance r = 0, 1, ... around the
-// query's cell are scanned; after ring r every unseen node is at least r*cs
-// away, so the search stops once the n_l-th distance is below (r cs)^2, or when
-// the whole periodic grid has been seen.
+// One warp per query.  The box of cells within Chebyshev distance r of the query's cell is
+// scanned row by row (the cells of a row are contiguous in the cell-sorted copies), r taken
+// from the number of nodes in the nearest 27 cells.  Every unseen node is then at least
+// r cs away, so the search ends once the n_l-th distance is below r cs, and otherwise goes
+// on with the shells r + 1, r + 2, ... until it is, or the whole periodic grid has been seen.
+//
+// A candidate costs a few FP32 operations: its FP32 distance is compared with the current
+// n_l-th distance plus 1e-6 (FP32 coordinates in [0, 1] put a distance off by less than
+// 4e-7), and only what passes gets the exact FP64 distance, 32 at a time, and is merged into
+// the 64 best, which the warp keeps sorted in registers (lane l: ranks l and 32 + l).  FP64
+// values compare as integers.  Measured: 86k queries of 40 (refined cloud) 1.14 ms in
+// place of 9.9 ms for one thread per query with its list in local memory, 616 wall queries of
+// 24 42 us in place of 1.03 ms.
+namespace {
+struct Best {
+    unsigned long long d[2];  // squared distance (bits), ranks lane and 32 + lane
+    int s[2];
+};
+__device__ __forceinline__ bool before(unsigned long long da, int sa, unsigned long long db, int sb,
+                                       const int32_t *perm) {
+    if (da != db) return da < db;
+    if (sa == sb || sa < 0 || sb < 0) return sa >= 0 && sb < 0;
+    return perm[sa] < perm[sb];
+}
+// compare-exchange with the lane `xor` away: the lower lane keeps the smaller when up
+__device__ __forceinline__ void exchange(unsigned long long &d, int &s, int mask, bool keep_small, const int32_t *perm) {
+    const unsigned long long od = __shfl_xor_sync(0xffffffffu, d, mask);
+    const int os = __shfl_xor_sync(0xffffffffu, s, mask);
+    if (before(od, os, d, s, perm) == keep_small) {
+        d = od;
+        s = os;
+    }
+}
+__device__ __forceinline__ void bitonic_merge(unsigned long long &d, int &s, int lane, const int32_t *perm) {
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) exchange(d, s, m, (lane & m) == 0, perm);
+}
+// the 64 best of 64 + 32 (one new entry per lane; absent: d all ones, s = -1)
+__device__ __forceinline__ void merge_in(Best &b, unsigned long long d, int s, int lane, const int32_t *perm) {
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int m = k >> 1; m > 0; m >>= 1) exchange(d, s, m, ((lane & m) == 0) == ((lane & k) == 0), perm);
+    // smaller halves of (ranks 32 .. 63) and (new, reversed), sorted
+    const unsigned long long rd = __shfl_xor_sync(0xffffffffu, d, 31);
+    const int rs = __shfl_xor_sync(0xffffffffu, s, 31);
+    if (before(rd, rs, b.d[1], b.s[1], perm)) {
+        b.d[1] = rd;
+        b.s[1] = rs;
+    }
+    bitonic_merge(b.d[1], b.s[1], lane, perm);
+    // the two sorted halves merged
+    const unsigned long long qd = __shfl_xor_sync(0xffffffffu, b.d[1], 31);
+    const int qs = __shfl_xor_sync(0xffffffffu, b.s[1], 31);
+    if (before(qd, qs, b.d[0], b.s[0], perm)) {
+        b.d[1] = b.d[0];
+        b.s[1] = b.s[0];
+        b.d[0] = qd;
+        b.s[0] = qs;
+    } else {
+        b.d[1] = qd;
+        b.s[1] = qs;
+    }
+    bitonic_merge(b.d[0], b.s[0], lane, perm);
+    bitonic_merge(b.d[1], b.s[1], lane, perm);
+}
+}  // namespace
+
 __global__ void __launch_bounds__(128) k_knn(int64_t nq, const double *__restrict__ qxyz,
                                              const int32_t *__restrict__ qnode, const double *__restrict__ xyz,
-                                             const int32_t *__restrict__ perm, const uint8_t *__restrict__ type,
-                                             int fluid_only, int G, const int32_t *__restrict__ cstart,
-                                             const int32_t *__restrict__ citems, int n_l, int32_t *out, int ld,
-                                             int col0, int32_t *status) {
-    int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+                                             const int32_t *__restrict__ perm, int fluid_only, int G,
+                                             const int32_t *__restrict__ cstart, const float4 *__restrict__ pts, int n_l,
+                                             int32_t *out, int ld, int col0, int32_t *status) {
+    __shared__ int pend[4][64];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t a = blockIdx.x * 4ll + warp;
     if (a >= nq) return;
-    double bd[RBF_MAX_NL];
-    int32_t bo[RBF_MAX_NL];
-    int32_t bs[RBF_MAX_NL];
-    int cnt = 0;
+    int *pd = pend[warp];
     double qx, qy, qz;
     if (qxyz) {
         qx = qxyz[3 * a]; qy = qxyz[3 * a + 1]; qz = qxyz[3 * a + 2];
@@ -290,56 +368,135 @@ __global__ void __launch_bounds__(128) k_knn(int64_t nq, const double *__restric
         qx = xyz[3 * s]; qy = xyz[3 * s + 1]; qz = xyz[3 * s + 2];
     }
     qx -= floor(qx); qy -= floor(qy); qz -= floor(qz);
+    const float fx = (float)qx, fy = (float)qy, fz = (float)qz;
     const double cs = 1.0 / G;
-    int cx = cell_coord(qx, G), cy = cell_coord(qy, G), cz = cell_coord(qz, G);
+    const int cx = cell_coord(qx, G), cy = cell_coord(qy, G), cz = cell_coord(qz, G);
     const int lo = -((G - 1) / 2), hi = G / 2;  // distinct periodic offsets
-    for (int r = 0;; ++r) {
-        bool any = false;
-        int ax0 = max(-r, lo), ax1 = min(r, hi);
-        for (int dx = ax0; dx <= ax1; ++dx)
-            for (int dy = ax0; dy <= ax1; ++dy)
-                for (int dz = ax0; dz <= ax1; ++dz) {
-                    int m = max(abs(dx), max(abs(dy), abs(dz)));
-                    if (m != r) continue;
-                    any = true;
-                    int ix = (cx + dx + G) % G, iy = (cy + dy + G) % G, iz = (cz + dz + G) % G;
-                    int64_t c = ((int64_t)ix * G + iy) * G + iz;
-                    int32_t e0 = cstart[c], e1 = cstart[c + 1];
-                    for (int32_t e = e0; e < e1; ++e) {
-                        int32_t s = citems[e];
-                        if (fluid_only && type[s]) continue;
-                        double ddx = mimg(xyz[3 * s] - qx);
-                        double ddy = mimg(xyz[3 * s + 1] - qy);
-                        double ddz = mimg(xyz[3 * s + 2] - qz);
-                        double d2 = dist2_nofma(ddx, ddy, ddz);
-                        int32_t o = perm[s];
-                        if (cnt == n_l && (d2 > bd[cnt - 1] || (d2 == bd[cnt - 1] && o > bo[cnt - 1]))) continue;
-                        int pos = cnt < n_l ? cnt++ : cnt - 1;
-                        while (pos > 0 && (bd[pos - 1] > d2 || (bd[pos - 1] == d2 && bo[pos - 1] > o))) {
-                            bd[pos] = bd[pos - 1]; bo[pos] = bo[pos - 1]; bs[pos] = bs[pos - 1];
-                            --pos;
-                        }
-                        bd[pos] = d2; bo[pos] = o; bs[pos] = s;
+    Best best;
+    best.d[0] = best.d[1] = ~0ull;
+    best.s[0] = best.s[1] = -1;
+    int n_pend = 0, seen = 0;
+    float thr = __int_as_float(0x7f800000);
+    auto kth = [&]() -> unsigned long long {
+        const unsigned long long v = n_l > 32 ? best.d[1] : best.d[0];
+        return __shfl_sync(0xffffffffu, v, (n_l - 1) & 31);
+    };
+    // exact distances of up to 32 pending candidates, merged into the best
+    auto flush = [&](int cnt) {
+        __syncwarp();
+        unsigned long long d = ~0ull;
+        int s = -1;
+        if (lane < cnt) {
+            s = pd[lane];
+            const double ddx = mimg(xyz[3 * (int64_t)s] - qx), ddy = mimg(xyz[3 * (int64_t)s + 1] - qy), ddz = mimg(xyz[3 * (int64_t)s + 2] - qz);
+            d = (unsigned long long)__double_as_longlong(dist2_nofma(ddx, ddy, ddz));
+        }
+        merge_in(best, d, s, lane, perm);
+        const unsigned long long k = kth();
+        if (k != ~0ull) {
+            const float r = sqrtf(__double2float_ru(__longlong_as_double((long long)k))) + 1e-6f;
+            thr = r * r * 1.000001f;
+        }
+        // what is left moves to the front
+        const int more = n_pend - cnt;
+        const int v = lane < more ? pd[cnt + lane] : 0;
+        __syncwarp();
+        if (lane < more) pd[lane] = v;
+        n_pend = more;
+        __syncwarp();
+    };
+    auto scan = [&](int e0, int e1) {
+        for (int base = e0; base < e1; base += 32) {
+            const int e = base + lane;
+            bool pass = false;
+            int s = 0;
+            if (e < e1) {
+                const float4 p = pts[e];
+                const uint32_t w = __float_as_uint(p.w);
+                float dx = p.x - fx, dy = p.y - fy, dz = p.z - fz;
+                dx -= rintf(dx); dy -= rintf(dy); dz -= rintf(dz);
+                s = (int)(w & 0x7fffffffu);
+                pass = dx * dx + dy * dy + dz * dz <= thr && !(fluid_only && (w >> 31));
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, pass);
+            if (m) {
+                if (pass) pd[n_pend + __popc(m & ((1u << lane) - 1u))] = s;
+                n_pend += __popc(m);
+                if (n_pend >= 32) flush(32);
+            }
+        }
+    };
+    // cells z0 .. z1 (offsets from the query's cell) of row (dx, dy)
+    auto row = [&](int dx, int dy, int z0, int z1, bool count_only) {
+        if (z0 > z1) return;
+        const int ix = (cx + dx + G) % G, iy = (cy + dy + G) % G;
+        const int32_t *c = cstart + ((int64_t)ix * G + iy) * G;
+        int i0 = cz + z0, i1 = cz + z1;
+        if (i1 < 0) { i0 += G; i1 += G; }
+        if (i0 >= G) { i0 -= G; i1 -= G; }
+        if (i0 < 0) {  // across the period: the end of the row, then its beginning
+            if (count_only) seen += c[G] - c[i0 + G];
+            else scan(c[i0 + G], c[G]);
+            i0 = 0;
+        }
+        if (i1 >= G) {
+            if (count_only) seen += c[i1 - G + 1] - c[0];
+            else scan(c[0], c[i1 - G + 1]);
+            i1 = G - 1;
+        }
+        if (i0 <= i1) {
+            if (count_only) seen += c[i1 + 1] - c[i0];
+            else scan(c[i0], c[i1 + 1]);
+        }
+    };
+    // boxes wider than the distinct offsets are cut to them
+    auto box = [&](int done, int r) {  // the cells at Chebyshev distance done + 1 .. r
+        const int x0 = max(-r, lo), x1 = min(r, hi);
+        for (int pass = 0; pass < 2; ++pass)  // the middle rows first: they fill the list with near nodes
+            for (int dx = x0; dx <= x1; ++dx)
+                for (int dy = x0; dy <= x1; ++dy) {
+                    const int m = max(abs(dx), abs(dy));
+                    if ((m <= 1) != (pass == 0)) continue;
+                    if (m > done) row(dx, dy, x0, x1, false);
+                    else {
+                        row(dx, dy, x0, min(x1, -done - 1), false);
+                        row(dx, dy, max(x0, done + 1), x1, false);
                     }
                 }
-        if (!any) break;  // every cell seen
-        double reach = r * cs;
-        if (cnt == n_l && bd[n_l - 1] < reach * reach * (1.0 - 1e-12)) break;
+    };
+    for (int dx = max(-1, lo); dx <= min(1, hi); ++dx)
+        for (int dy = max(-1, lo); dy <= min(1, hi); ++dy) row(dx, dy, max(-1, lo), min(1, hi), true);
+    // radius (in cells) of a ball with n_l nodes at the density of the nearest 27 cells
+    int r = max(1, (int)ceilf(1.1f * cbrtf((float)n_l * 27.0f / (4.19f * (float)max(seen, 1)))));
+    int done = -1;
+    for (;;) {
+        r = min(r, G);
+        box(done, r);
+        while (n_pend > 0) flush(min(n_pend, 32));
+        if (-r <= lo && r >= hi) break;  // every cell seen
+        const double reach = r * cs;
+        const unsigned long long k = kth();
+        if (k != ~0ull && __longlong_as_double((long long)k) < reach * reach * (1.0 - 1e-12)) break;
+        done = r;
+        ++r;
     }
-    if (cnt < n_l) {
-        atomicExch(status, 1);
-        for (int t = cnt; t < n_l; ++t) bs[t] = cnt > 0 ? bs[0] : 0;  // flagged: never used
+    const unsigned have = __popc(__ballot_sync(0xffffffffu, best.s[0] >= 0)) + __popc(__ballot_sync(0xffffffffu, best.s[1] >= 0));
+    if ((int)have < n_l) {
+        if (lane == 0) atomicExch(status, 1);
+        const int s0 = max(__shfl_sync(0xffffffffu, best.s[0], 0), 0);
+        for (int h = 0; h < 2; ++h)
+            if (best.s[h] < 0) best.s[h] = s0;  // flagged: never used
     }
-    for (int t = 0; t < n_l; ++t) out[a * ld + col0 + t] = bs[t];
+    for (int h = 0; h < 2; ++h)
+        if (lane + 32 * h < n_l) out[a * ld + col0 + lane + 32 * h] = best.s[h];
 }
 
-cudaError_t launch_knn(int64_t nq, const double *qxyz, const int32_t *qnode, const double *xyz,
-                       const int32_t *perm, const uint8_t *type, int fluid_only, int G,
-                       const int32_t *cell_start, const int32_t *cell_items, int n_l, int32_t *out, int ld,
-                       int col0, int32_t *status, cudaStream_t st) {
+cudaError_t launch_knn(int64_t nq, const double *qxyz, const int32_t *qnode, const double *xyz, const int32_t *perm,
+                       int fluid_only, int G, const int32_t *cell_start, const float4 *pts, int n_l, int32_t *out,
+                       int ld, int col0, int32_t *status, cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
-    k_knn<<<(unsigned)((nq + 127) / 128), 128, 0, st>>>(nq, qxyz, qnode, xyz, perm, type, fluid_only, G,
-                                                        cell_start, cell_items, n_l, out, ld, col0, status);
+    k_knn<<<(unsigned)((nq + 3) / 4), 128, 0, st>>>(nq, qxyz, qnode, xyz, perm, fluid_only, G, cell_start, pts, n_l, out,
+                                                    ld, col0, status);
     return cudaGetLastError();
 }
 
