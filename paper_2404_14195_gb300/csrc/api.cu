@@ -603,12 +603,14 @@ int compute_weights_impl(rbf_ctx *ctx, int phs_k, int mono_m, int solver, int q,
     CK(cudaMemcpyAsync(d_gops.p, gops.data(), 3 * sizeof(OpSpec), cudaMemcpyHostToDevice, ctx->st));
     if (presolved && solver != RBF_SOLVER_ACM) return fail(ctx, RBF_EINVAL, "presolved weights: ACM only");
     CK(ctx->status.zero(ctx->st));
+    DevArr<int32_t> list;  // systems handed from the FP32 to the FP64 factors
+    CK(list.alloc(n + 1));
     if (!presolved) {
         CK(ctx->w64.alloc(n * n_ops * n_l));
         CK(ctx->delta.alloc(n));
         CK(launch_weights(n, ctx->xyz.p, nullptr, ctx->iota.p, 1, n_l, ctx->idx.p, phs_k, mono_m, n_ops, d_ops.p,
-                          ctx->w64.p, ctx->delta.p, ctx->status.p, ctx->st));
-        ++ctx->launches;
+                          ctx->w64.p, ctx->delta.p, ctx->status.p, list.p, ctx->st));
+        ctx->launches += phs_k > 5 ? 1 : 2;
         CK(ctx->wgb64.alloc(nb * 3 * n_l));
     }
     CK(ctx->wgw64.alloc(nb * 3 * n_l));
@@ -618,12 +620,12 @@ int compute_weights_impl(rbf_ctx *ctx, int phs_k, int mono_m, int solver, int q,
             ++ctx->launches;
             if (!presolved)
                 CK(launch_weights(nb, ctx->xyz.p, nullptr, ctx->wall.p, 1, n_l, ctx->idxb.p, phs_k, mono_m, 3, d_gops.p,
-                                  ctx->wgb64.p, nullptr, ctx->status.p + 1, ctx->st));
+                                  ctx->wgb64.p, nullptr, ctx->status.p + 1, list.p, ctx->st));
         } else {
             CK(launch_weights(nb, ctx->xyz.p, nullptr, ctx->wall.p, 1, n_l, ctx->idxw.p, phs_k, mono_m, 3, d_gops.p,
-                              ctx->wgw64.p, nullptr, ctx->status.p + 1, ctx->st));
+                              ctx->wgw64.p, nullptr, ctx->status.p + 1, list.p, ctx->st));
         }
-        ++ctx->launches;
+        ctx->launches += phs_k > 5 ? 1 : 2;
     }
     if (ctx->partial.n < (size_t)(4 * (nblk(n) + 8))) CK(ctx->partial.alloc(4 * (nblk(n) + 8)));
     CK(launch_min_f64(ctx->delta.p, n, ctx->partial.p, ctx->scal.p, ctx->st));
@@ -1194,7 +1196,7 @@ int ensure_probes(rbf_ctx *ctx, int m_p) {
     const int64_t tot = 5LL * m_p * m_p;
     const int n_l = ctx->n_l;
     DevArr<double> pts, pxyz, pw;
-    DevArr<int32_t> flag, scan, tmp, pidx;
+    DevArr<int32_t> flag, scan, tmp, pidx, list;
     CK(pts.alloc(3 * tot)); CK(flag.alloc(tot + 1)); CK(scan.alloc(tot + 1)); CK(tmp.alloc(scan_tmp_len(tot + 1)));
     CK(flag.zero(ctx->st));
     k_probe_points<<<nblk(tot), 256, 0, ctx->st>>>(m_p, ctx->c[0], ctx->c[1], ctx->c[2], ctx->r, ctx->has_sphere, pts.p, flag.p);
@@ -1212,10 +1214,11 @@ int ensure_probes(rbf_ctx *ctx, int m_p) {
         CK(launch_knn(nfl, pxyz.p, nullptr, ctx->xyz.p, ctx->perm.p, 0, ctx->G, ctx->cstart.p, ctx->cpts.p, n_l, pidx.p, n_l, 0, ctx->status.p, ctx->st));
         OpSpec op{OP_INTERP, {0.0, 0.0, 0.0}};
         DevArr<OpSpec> d_op;
+        CK(list.alloc((int64_t)nfl + 1));
         CK(d_op.alloc(1));
         CK(cudaMemcpyAsync(d_op.p, &op, sizeof(OpSpec), cudaMemcpyHostToDevice, ctx->st));
         CK(launch_weights(nfl, ctx->xyz.p, pxyz.p, nullptr, 0, n_l, pidx.p, ctx->phs_k, ctx->mono_m, 1,
-                          d_op.p, pw.p, nullptr, ctx->status.p + 1, ctx->st));
+                          d_op.p, pw.p, nullptr, ctx->status.p + 1, list.p, ctx->st));
         ctx->launches += 2;
     }
     int32_t st2[2] = {0, 0};
@@ -1795,20 +1798,21 @@ int rbf_batch_build(rbf_batch *b, int phs_k, int mono_m, rbf_weight_report *rep)
     DevArr<WeightJob> dj, dwj;
     DevArr<int64_t> dpn, dpw;
     DevArr<OpSpec> dops, dgops;
-    DevArr<int32_t> dsing;
+    DevArr<int32_t> dsing, dlist;
+    CK(dlist.alloc(std::max(pn[nc], pw.back()) + 1));
     CK(dj.alloc(nc)); CK(dpn.alloc(nc + 1)); CK(dops.alloc(4)); CK(dgops.alloc(3)); CK(dsing.alloc(2));
     CK(cudaMemcpyAsync(dj.p, nodes.data(), nc * sizeof(WeightJob), cudaMemcpyHostToDevice, b->st));
     CK(cudaMemcpyAsync(dpn.p, pn.data(), (nc + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, b->st));
     CK(cudaMemcpyAsync(dops.p, ops.data(), 4 * sizeof(OpSpec), cudaMemcpyHostToDevice, b->st));
     CK(cudaMemcpyAsync(dgops.p, gops.data(), 3 * sizeof(OpSpec), cudaMemcpyHostToDevice, b->st));
     CK(dsing.zero(b->st));
-    CK(launch_weights_multi(nc, dj.p, dpn.p, pn[nc], max_nl, phs_k, mono_m, 4, dops.p, dsing.p, b->st));
+    CK(launch_weights_multi(nc, dj.p, dpn.p, pn[nc], max_nl, phs_k, mono_m, 4, dops.p, dsing.p, dlist.p, b->st));
     if (!walls.empty()) {
         CK(dwj.alloc(walls.size())); CK(dpw.alloc(pw.size()));
         CK(cudaMemcpyAsync(dwj.p, walls.data(), walls.size() * sizeof(WeightJob), cudaMemcpyHostToDevice, b->st));
         CK(cudaMemcpyAsync(dpw.p, pw.data(), pw.size() * sizeof(int64_t), cudaMemcpyHostToDevice, b->st));
         CK(launch_weights_multi((int)walls.size(), dwj.p, dpw.p, pw.back(), max_nl, phs_k, mono_m, 3, dgops.p,
-                                dsing.p + 1, b->st));
+                                dsing.p + 1, dlist.p, b->st));
     }
     int32_t sing[2] = {0, 0};
     CK(cudaMemcpyAsync(sing, dsing.p, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, b->st));

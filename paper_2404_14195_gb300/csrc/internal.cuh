@@ -76,10 +76,11 @@ cudaError_t launch_knn(int64_t nq, const double *qxyz, const int32_t *qnode, con
                        int fluid_only, int G, const int32_t *cell_start, const float4 *pts, int n_l, int32_t *out,
                        int ld, int col0, int32_t *status, cudaStream_t st);
 
-// weights.cu
+// weights.cu; list: device scratch, one int32 per system and one more
 cudaError_t launch_weights(int64_t nc, const double *xyz, const double *cxyz, const int32_t *cnode,
                            int centre_is_node, int n_l, const int32_t *idx, int k, int m, int n_ops,
-                           const OpSpec *ops, double *w, double *delta, int32_t *n_sing, cudaStream_t st);
+                           const OpSpec *ops, double *w, double *delta, int32_t *n_sing, int32_t *list,
+                           cudaStream_t st);
 
 // one entry of a multi-set weight launch: nc centres, centre c = node cnode[c] of
 // xyz with stencil idx[c * n_l ..] -> w[(c * n_ops + o) * n_l + j], delta[c]
@@ -93,7 +94,7 @@ struct WeightJob {
     double *delta;
 };
 cudaError_t launch_weights_multi(int njobs, const WeightJob *jobs_dev, const int64_t *prefix_dev, int64_t ntot,
-                                 int max_n_l, int k, int m, int n_ops, const OpSpec *ops, int32_t *n_sing,
+                                 int max_n_l, int k, int m, int n_ops, const OpSpec *ops, int32_t *n_sing, int32_t *list,
                                  cudaStream_t st);
 
 // pack.cu (in weights.cu): FP64 row weights [c][o][j] -> SELL T [s][o][j][lane]
