@@ -272,7 +272,8 @@ int rbf_profile_steps(rbf_ctx *ctx, int nsteps, double *kernel_ms, int *n_classe
  * mapping of the ACM sweeps of rbf_step instead: block + 1000 G, with block =
  * 64, 128 or 256 threads and G = 2 or 4 lanes per node, each lane summing every
  * G-th stencil column (write 0 for one lane per node, i.e. the code is the block
- * size; default 256).  RBF_EINVAL for any other code. */
+ * size; until it is set, by the number of nodes: four lanes, then two, then
+ * 256).  RBF_EINVAL for any other code. */
 int rbf_set_kernel_variant(rbf_ctx *ctx, int variant);
 
 #define RBF_TUNE_MAX 16

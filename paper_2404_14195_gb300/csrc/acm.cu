@@ -230,14 +230,19 @@ __global__ void k_acm_vmax(AcmArgs<T> a, int slot) {
     if ((threadIdx.x & 31) == 0 && sp > 0.0) atomicMax(a.vmax + slot, (unsigned long long)__double_as_longlong(sp));
 }
 
+// Lanes per node of the wall sweep: wall nodes are few (60k of 600k) and one lane's 25 dependent
+// gathers are the sweep's time, so four lanes share them at every schedule (FP32 step of 600k
+// nodes 586 -> 571 us; one lane per wall node 18.8 us of each of its three wall sweeps).
+constexpr int WALL_LANES = 4;
+
 // Iteration g of the run (counted over all steps) writes max |v| into slot g % 2;
 // the pressure sweep of iteration g reads slot (g + 1) % 2 (the previous
 // iteration's) and clears slot g % 2 for its own correction sweep.  The grids
-// cover every slice with G warps per slice.
+// cover every slice with G warps per slice, the wall sweep's with WALL_LANES.
 template <typename T, bool CP, int G>
 cudaError_t acm_launch_step_g(const AcmArgs<T> &a, int n_p, int parity, cudaStream_t st, int64_t *launches,
                               LaunchRecorder *rec, int block) {
-    const int64_t threads = ((a.n + 31) >> 5) * 32 * G, threads_b = ((a.nb + 31) >> 5) * 32 * G;
+    const int64_t threads = ((a.n + 31) >> 5) * 32 * G, threads_b = ((a.nb + 31) >> 5) * 32 * WALL_LANES;
     const unsigned gb = (unsigned)((threads + block - 1) / block);
     const unsigned gw = (unsigned)((threads_b + 255) / 256);
     if (rec) rec->begin(st, 0);
@@ -255,7 +260,7 @@ cudaError_t acm_launch_step_g(const AcmArgs<T> &a, int n_p, int parity, cudaStre
         ++*launches;
         if (a.nb > 0) {
             if (rec) rec->begin(st, 2);
-            k_acm_wall_pressure<T, CP, G><<<gw, 256, 0, st>>>(a);
+            k_acm_wall_pressure<T, CP, WALL_LANES><<<gw, 256, 0, st>>>(a);
             if (rec) rec->end(st);
             ++*launches;
         }

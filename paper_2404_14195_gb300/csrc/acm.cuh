@@ -58,6 +58,19 @@ inline bool acm_code_ok(int code) {
     return code > 0 && (block == 64 || block == 128 || block == 256) && (group == 0 || group == 2 || group == 4);
 }
 
+// The code for n nodes when the caller has set none.  One lane per node leaves a small cell
+// with few warps, each walking n_l dependent gathers; more lanes shorten that walk until the
+// chip is full (FP64: until its pipe is).  us per step with 1 / 2 / 4 lanes, N_L = 25, GB300:
+//   FP64  944 nodes 117 / 83 / 75, 6k 115 / 88 / 86, 18k 117 / 97 / 107, 49k 201 / 172 / 209,
+//         112k 262 / 305 / 394
+//   FP32  944 nodes 70 / 67 / 55, 18k 78 / 71 / 65, 49k 142 / 110 / 95, 112k 148 / 130 / 153,
+//         257k 265 / 266 / 285
+// The lines lie between, in nodes per SM.
+inline int acm_code_auto(int64_t n, int sms, bool fp64) {
+    const int64_t four = fp64 ? 64 : 448, two = fp64 ? 448 : 1024;
+    return n <= sms * four ? 4128 : n <= sms * two ? 2128 : 256;
+}
+
 template <typename T>
 cudaError_t acm_launch_step(const AcmArgs<T> &a, int n_p, int parity, cudaStream_t st, int64_t *launches,
                             LaunchRecorder *rec = nullptr, int code = 256);

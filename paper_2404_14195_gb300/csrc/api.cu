@@ -272,8 +272,9 @@ cudaError_t enqueue_steps(rbf_ctx *ctx, int steps, int &parity, int &cur, int64_
             continue;
         }
         if (ctx->solver == RBF_SOLVER_ACM) {
-            if (is_f32(ctx)) e = acm_launch_step<float>(acm_args<float>(ctx, ctx->a32, ctx->ws32, ctx->wn32), ctx->n_p, parity, ctx->st, launches, rec, ctx->acm_code);
-            else e = acm_launch_step<double>(acm_args<double>(ctx, ctx->a64, ctx->ws64, ctx->wn64), ctx->n_p, parity, ctx->st, launches, rec, ctx->acm_code);
+            const int code = ctx->acm_code ? ctx->acm_code : acm_code_auto(ctx->n, ctx->sms, !is_f32(ctx));
+            if (is_f32(ctx)) e = acm_launch_step<float>(acm_args<float>(ctx, ctx->a32, ctx->ws32, ctx->wn32), ctx->n_p, parity, ctx->st, launches, rec, code);
+            else e = acm_launch_step<double>(acm_args<double>(ctx, ctx->a64, ctx->ws64, ctx->wn64), ctx->n_p, parity, ctx->st, launches, rec, code);
             parity = (parity + ctx->n_p) & 1;
         } else {
             if (rec) rec->begin(ctx->st, 0);

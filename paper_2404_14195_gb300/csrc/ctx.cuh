@@ -103,7 +103,7 @@ struct rbf_ctx {
     int variant = rbf::LBM_RECORD_PER_THREAD_PDL;  // schedule of the fused LBM step
     bool variant_auto = true;                      // not set by the caller: chosen by size in rbf_init
     int lbm_layout = rbf::LBM_LAYOUT_NODES;  // layout of f32 / f64 (follows the schedule)
-    int acm_code = 256;               // ACM sweeps: threads per block + 1000 x lanes per node (0: one)
+    int acm_code = 0;                 // ACM sweeps: threads per block + 1000 x lanes per node (0: one); 0: by size
     int persist_block = 0;            // threads per block of the persistent ACM driver (0: chosen by size)
     int persist_cluster = 0;          // > 0: run it as one cluster of that many CTAs (8 or 16)
     int persist_group = 1;            // lanes per node of its sweeps (1, 2, 4, 8)
