@@ -16,8 +16,8 @@
 // stencil index -> gathered field -> sum -> barrier decides.
 //  * One cell whose stencils fit the SMs' shared memory (34 MB on the chip: about 30k
 //    nodes at N_L = 25 in FP64, 55k in FP32) runs resident, k_acm_resident below.
-//  * Everything else streams its stencils, k_acm_persistent, with the cells'
-//    descriptors and done flags in shared memory.
+//  * Everything else streams its stencils, k_acm_persistent, with the cells' unit counts
+//    and done flags in shared memory.
 //  * The barrier is one monotonic counter: one release-add per block, polling
 //    acquire loads, no reset.
 //
@@ -282,13 +282,14 @@ __device__ __forceinline__ T phase_correct(const CellDesc<T> &c, const Sten<T> s
 // synchronised by the cluster's hardware barrier.  Every block of a cluster takes the
 // same branches at every barrier (the done flags change only before a barrier and
 // the cluster barrier cannot time out), so none is left waiting.  Dynamic shared
-// memory: descriptors, unit counts, residual sums and flags of the cells.
+// memory: residual sums, unit counts and flags of the cells.  The descriptors stay in global
+// memory: 250 bytes of each cell in every block take the L1 from the gathers (64 cells, 7.3M
+// nodes, FP32: 6.55 ms per step with copies in shared memory, 5.73 ms without).
 template <typename T, bool CP, bool CL, int G>
-__global__ void __launch_bounds__(256) k_acm_persistent(const CellDesc<T> *__restrict__ cells_g, PersistCtl ctl) {
+__global__ void __launch_bounds__(256) k_acm_persistent(const CellDesc<T> *__restrict__ cells, PersistCtl ctl) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int nc = ctl.ncells;
-    CellDesc<T> *cells = reinterpret_cast<CellDesc<T> *>(sm);
-    double *racc = reinterpret_cast<double *>(cells + nc);  // [nc][2]
+    double *racc = reinterpret_cast<double *>(sm);              // [nc][2]
     int64_t *pre = reinterpret_cast<int64_t *>(racc + 2 * nc);  // [nc + 1] units ahead of each cell
     int64_t *wpre = pre + nc + 1;                               // [nc + 1] wall units
     int *done = reinterpret_cast<int *>(wpre + nc + 1);         // [nc]
@@ -299,17 +300,18 @@ __global__ void __launch_bounds__(256) k_acm_persistent(const CellDesc<T> *__res
     constexpr int NU = 32 / G;  // nodes per unit
 
     {
-        const int words = nc * (int)(sizeof(CellDesc<T>) / 4);
-        for (int e = threadIdx.x; e < words; e += blockDim.x)
-            reinterpret_cast<int *>(cells)[e] = reinterpret_cast<const int *>(cells_g)[e];
-        for (int c = threadIdx.x; c < nc; c += blockDim.x) done[c] = 0;
+        for (int c = threadIdx.x; c < nc; c += blockDim.x) {
+            done[c] = 0;
+            pre[c + 1] = ((cells[c].n + 31) >> 5) * G;
+            wpre[c + 1] = ((cells[c].nb + 31) >> 5) * G;
+        }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         pre[0] = wpre[0] = 0;
         for (int c = 0; c < nc; ++c) {
-            pre[c + 1] = pre[c] + ((cells[c].n + 31) >> 5) * G;
-            wpre[c + 1] = wpre[c] + ((cells[c].nb + 31) >> 5) * G;
+            pre[c + 1] += pre[c];
+            wpre[c + 1] += wpre[c];
         }
     }
     __syncthreads();

@@ -45,11 +45,11 @@ struct PersistCtl {
     unsigned long long *vsq; // resident kernel: 2 slots of max |v|^2
 };
 
-// shared memory of the streaming kernel: descriptors, residual accumulators, unit
-// counts ahead of each cell, flags
+// shared memory of the streaming kernel: residual accumulators, unit counts ahead of each
+// cell, flags
 template <typename T>
 __host__ __device__ constexpr int64_t persist_head_bytes(int ncells) {
-    return ((int64_t)ncells * (int64_t)sizeof(CellDesc<T>) + (ncells + 1) * 16ll + ncells * 16ll + ncells * 4ll + 15) & ~15ll;
+    return ((ncells + 1) * 16ll + ncells * 16ll + ncells * 4ll + 15) & ~15ll;
 }
 // Shares of the resident kernel (one cell, every block's stencils in shared memory):
 // largest number of units and wall units per block, local nodes there is room for,
