@@ -282,14 +282,18 @@ __device__ __forceinline__ T phase_correct(const CellDesc<T> &c, const Sten<T> s
 // synchronised by the cluster's hardware barrier.  Every block of a cluster takes the
 // same branches at every barrier (the done flags change only before a barrier and
 // the cluster barrier cannot time out), so none is left waiting.  Dynamic shared
-// memory: residual sums, unit counts and flags of the cells.  The descriptors stay in global
-// memory: 250 bytes of each cell in every block take the L1 from the gathers (64 cells, 7.3M
-// nodes, FP32: 6.55 ms per step with copies in shared memory, 5.73 ms without).
-template <typename T, bool CP, bool CL, int G>
-__global__ void __launch_bounds__(256) k_acm_persistent(const CellDesc<T> *__restrict__ cells, PersistCtl ctl) {
+// memory: residual sums, unit counts and flags of the cells.  SH: the descriptors of up to
+// PERSIST_SHARED_CELLS cells are copied there too; with more the copies, 250 bytes a cell in
+// every block, take the L1 from the gathers (FP32: 12 cells, 105 steps 51.3 ms with copies, 52.5
+// without; 64 cells, 7.3M nodes 6.55 ms per step with, 5.73 without).
+template <typename T, bool CP, bool CL, int G, bool SH>
+__global__ void __launch_bounds__(256) k_acm_persistent(const CellDesc<T> *__restrict__ cells_g, PersistCtl ctl) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int nc = ctl.ncells;
-    double *racc = reinterpret_cast<double *>(sm);              // [nc][2]
+    CellDesc<T> *own = reinterpret_cast<CellDesc<T> *>(sm);
+    const CellDesc<T> *cells;
+    if constexpr (SH) cells = own; else cells = cells_g;
+    double *racc = reinterpret_cast<double *>(own + (SH ? nc : 0));  // [nc][2]
     int64_t *pre = reinterpret_cast<int64_t *>(racc + 2 * nc);  // [nc + 1] units ahead of each cell
     int64_t *wpre = pre + nc + 1;                               // [nc + 1] wall units
     int *done = reinterpret_cast<int *>(wpre + nc + 1);         // [nc]
@@ -300,10 +304,15 @@ __global__ void __launch_bounds__(256) k_acm_persistent(const CellDesc<T> *__res
     constexpr int NU = 32 / G;  // nodes per unit
 
     {
+        if constexpr (SH) {
+            const int words = nc * (int)(sizeof(CellDesc<T>) / 4);
+            for (int e = threadIdx.x; e < words; e += blockDim.x)
+                reinterpret_cast<int *>(own)[e] = reinterpret_cast<const int *>(cells_g)[e];
+        }
         for (int c = threadIdx.x; c < nc; c += blockDim.x) {
             done[c] = 0;
-            pre[c + 1] = ((cells[c].n + 31) >> 5) * G;
-            wpre[c + 1] = ((cells[c].nb + 31) >> 5) * G;
+            pre[c + 1] = ((cells_g[c].n + 31) >> 5) * G;
+            wpre[c + 1] = ((cells_g[c].nb + 31) >> 5) * G;
         }
     }
     __syncthreads();
@@ -950,23 +959,26 @@ const void *resident_kernel(int group) {
 
 bool persist_block_ok(int block) { return block == 32 || block == 64 || block == 128 || block == 256; }
 
-template <typename T, bool CP>
+template <typename T, bool CP, bool SH>
 const void *grid_kernel(int group) {
     switch (group) {
-    case 1: return (const void *)k_acm_persistent<T, CP, false, 1>;
-    case 2: return (const void *)k_acm_persistent<T, CP, false, 2>;
-    case 4: return (const void *)k_acm_persistent<T, CP, false, 4>;
-    case 8: return (const void *)k_acm_persistent<T, CP, false, 8>;
+    case 1: return (const void *)k_acm_persistent<T, CP, false, 1, SH>;
+    case 2: return (const void *)k_acm_persistent<T, CP, false, 2, SH>;
+    case 4: return (const void *)k_acm_persistent<T, CP, false, 4, SH>;
+    case 8: return (const void *)k_acm_persistent<T, CP, false, 8, SH>;
     default: return nullptr;
     }
 }
 template <typename T>
-const void *grid_kernel(int group, bool cp) { return cp ? grid_kernel<T, true>(group) : grid_kernel<T, false>(group); }
+const void *grid_kernel(int group, bool cp, bool sh) {
+    if (sh) return cp ? grid_kernel<T, true, true>(group) : grid_kernel<T, false, true>(group);
+    return cp ? grid_kernel<T, true, false>(group) : grid_kernel<T, false, false>(group);
+}
 
 template <typename T, bool CP>
 cudaError_t launch_cluster_T(const CellDesc<T> *cells_dev, const PersistCtl &ctl, int csize, size_t smem, cudaStream_t st,
                              int *max_clusters) {
-    auto kern = k_acm_persistent<T, CP, true, 1>;
+    auto kern = k_acm_persistent<T, CP, true, 1, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -992,7 +1004,7 @@ cudaError_t launch_cluster_T(const CellDesc<T> *cells_dev, const PersistCtl &ctl
 template <typename T>
 cudaError_t acm_launch_persistent(const CellDesc<T> *cells_dev, const PersistCtl &ctl, int nblocks, int block,
                                   int group, bool cp, cudaStream_t st) {
-    const void *fn = grid_kernel<T>(group, cp);
+    const void *fn = grid_kernel<T>(group, cp, ctl.ncells <= PERSIST_SHARED_CELLS);
     if (!persist_block_ok(block) || nblocks < 1 || !fn) return cudaErrorInvalidValue;
     const size_t smem = persist_head_bytes<T>(ctl.ncells);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1026,8 +1038,9 @@ cudaError_t acm_persistent_cluster_ok(int csize, bool cp, size_t smem, bool *ok)
 }
 
 template <typename T>
-cudaError_t acm_persistent_max_blocks(int *blocks, int block, int group, bool cp, size_t smem) {
-    const void *fn = grid_kernel<T>(group, cp);
+cudaError_t acm_persistent_max_blocks(int *blocks, int block, int group, bool cp, int ncells) {
+    const size_t smem = persist_head_bytes<T>(ncells);
+    const void *fn = grid_kernel<T>(group, cp, ncells <= PERSIST_SHARED_CELLS);
     if (!persist_block_ok(block) || !fn) return cudaErrorInvalidValue;
     int dev = 0, sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1073,7 +1086,7 @@ cudaError_t acm_launch_resident(const CellDesc<T> &cell, const PersistCtl &ctl, 
 #define RBF_PERSIST_INST(T)                                                                                            \
     template cudaError_t acm_launch_persistent<T>(const CellDesc<T> *, const PersistCtl &, int, int, int, bool,        \
                                                   cudaStream_t);                                                       \
-    template cudaError_t acm_persistent_max_blocks<T>(int *, int, int, bool, size_t);                                  \
+    template cudaError_t acm_persistent_max_blocks<T>(int *, int, int, bool, int);                                  \
     template cudaError_t acm_launch_persistent_cluster<T>(const CellDesc<T> *, const PersistCtl &, int, bool,          \
                                                           cudaStream_t);                                               \
     template cudaError_t acm_persistent_cluster_ok<T>(int, bool, size_t, bool *);                                      \

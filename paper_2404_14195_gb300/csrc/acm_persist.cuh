@@ -45,11 +45,13 @@ struct PersistCtl {
     unsigned long long *vsq; // resident kernel: 2 slots of max |v|^2
 };
 
-// shared memory of the streaming kernel: residual accumulators, unit counts ahead of each
+// cells whose descriptors the streaming kernel copies to shared memory
+constexpr int PERSIST_SHARED_CELLS = 16;
+// shared memory of the streaming kernel: descriptors, residual accumulators, unit counts ahead of each
 // cell, flags
 template <typename T>
 __host__ __device__ constexpr int64_t persist_head_bytes(int ncells) {
-    return ((ncells + 1) * 16ll + ncells * 16ll + ncells * 4ll + 15) & ~15ll;
+    return ((ncells <= PERSIST_SHARED_CELLS ? ncells : 0) * (int64_t)sizeof(CellDesc<T>) + (ncells + 1) * 16ll + ncells * 16ll + ncells * 4ll + 15) & ~15ll;
 }
 // Shares of the resident kernel (one cell, every block's stencils in shared memory):
 // largest number of units and wall units per block, local nodes there is room for,
@@ -74,7 +76,7 @@ cudaError_t acm_launch_persistent(const CellDesc<T> *cells_dev, const PersistCtl
                                   int group, bool cp, cudaStream_t st);
 // co-resident blocks of the kernel with `smem` bytes of dynamic shared memory each
 template <typename T>
-cudaError_t acm_persistent_max_blocks(int *blocks, int block, int group, bool cp, size_t smem);
+cudaError_t acm_persistent_max_blocks(int *blocks, int block, int group, bool cp, int ncells);
 // the same kernel as one thread-block cluster of csize (8 or 16) CTAs of 256
 // threads, synchronised by the cluster barrier
 template <typename T>

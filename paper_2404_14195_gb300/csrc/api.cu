@@ -1406,7 +1406,7 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
     // blocks and the share of the last round's warps that have a unit
     auto grid = [&](int block, int group, int *nblocks) -> double {
         int maxb = 0;
-        p.err = acm_persistent_max_blocks<T>(&maxb, block, group, cp, (size_t)persist_head_bytes<T>((int)cs.size()));
+        p.err = acm_persistent_max_blocks<T>(&maxb, block, group, cp, (int)cs.size());
         const int64_t wpb = block / 32, units = slices * group;
         *nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(maxb, (units + wpb - 1) / wpb));
         const double rounds = (double)units / ((double)*nblocks * wpb);
