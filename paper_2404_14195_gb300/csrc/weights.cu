@@ -21,7 +21,7 @@
 //    slices relative to the row's (column's) largest exponent, six to eight 32 x 32 -> 64
 //    bit multiply-adds per product accumulate exactly.  A compensated FP64 dot product (ten
 //    FP64 operations per product) was two thirds of the FP64 work of an 18-operator system.
-//  * One reciprocal per pivot instead of a division per row and right-hand side; each
+//  * One reciprocal per pivot instead of a division per right-hand side; each
 //    distance of the symmetric A computed once.
 //  * FP64 updates run over (row, column) pairs packed over the block's threads with
 //    incremental indices (no integer division), so warps stay full at small sizes.
@@ -420,7 +420,10 @@ __device__ void weights_fp64(int64_t c, double *sm, const WJob &J) {
     __syncthreads();
     // LU with partial pivoting (rows swapped in full, multipliers stored below).  Every
     // warp finds the pivot for itself: magnitudes compared as integers, not-a-numbers
-    // passed over, ties to the smaller row.
+    // passed over, ties to the smaller row.  The multipliers are quotients: of two equal
+    // rows the second becomes exactly zero and the system is found singular, whereas
+    // a * (1 / a) is 1 - 2^-53 for one pivot in seven (18 to 37 of 253 to 503 systems with
+    // two coincident nodes then passed).
     bool singular = false;
     for (int col = 0; col < ns; ++col) {
         long long best = -1;
@@ -446,7 +449,7 @@ __device__ void weights_fp64(int64_t c, double *sm, const WJob &J) {
                     M[col * ld + q] = M[bi * ld + q];
                     M[bi * ld + q] = s;
                 }
-        for (int r = col + 1 + (WT - 1 - t); r < ns; r += WT) M[r * ld + col] = (r == bi ? dv : M[r * ld + col]) * inv;
+        for (int r = col + 1 + (WT - 1 - t); r < ns; r += WT) M[r * ld + col] = (r == bi ? dv : M[r * ld + col]) / pv;
         if (t == WT - 1) {
             M[col * ld + col] = pv;
             rp[col] = inv;
