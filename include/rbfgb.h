@@ -321,6 +321,17 @@ int rbf_autotune_persistent(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep)
  * the order of the stencil sums (rounding only). */
 int rbf_set_persistent_block(rbf_ctx *ctx, int code);
 
+/* The schedule that the last persistent launch of this context (a batch: of its first
+ * cell) ran with.  RBF_EINVAL before the first one. */
+typedef struct {
+    int32_t resident;  /* 1: one cell, stencils in the SMs' shared memory */
+    int32_t cluster;   /* CTAs of the cluster; 0: a cooperative grid */
+    int32_t threads;   /* per block */
+    int32_t lanes;     /* per node */
+    int32_t blocks;
+} rbf_persist_info;
+int rbf_persistent_info(rbf_ctx *ctx, rbf_persist_info *info);
+
 /* Wall-clock limit of one wait at a grid barrier of the persistent ACM driver
  * (rbf_solve, rbf_batch_solve with this context as the first cell): a block that
  * waits longer for the others raises the launch's error flag, every block leaves

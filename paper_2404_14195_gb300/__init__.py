@@ -55,6 +55,10 @@ class rbf_tune_report(ctypes.Structure):
                 ("ms_per_step", ctypes.c_double * 16), ("chosen", ctypes.c_int)]
 
 
+class rbf_persist_info(ctypes.Structure):
+    _fields_ = [(f, ctypes.c_int32) for f in ("resident", "cluster", "threads", "lanes", "blocks")]
+
+
 class rbf_batch_cell_result(ctypes.Structure):
     _fields_ = [("steps", ctypes.c_int64), ("residual", ctypes.c_double), ("k_over_d2", ctypes.c_double),
                 ("status", ctypes.c_int)]
@@ -106,6 +110,7 @@ ABI = {
     "rbf_autotune": (_I, [_P, _I, ctypes.POINTER(rbf_tune_report)]),
     "rbf_autotune_persistent": (_I, [_P, _I, ctypes.POINTER(rbf_tune_report)]),
     "rbf_set_persistent_block": (_I, [_P, _I]),
+    "rbf_persistent_info": (_I, [_P, ctypes.POINTER(rbf_persist_info)]),
     "rbf_set_wait_limit": (_I, [_P, _D]),
     "rbf_batch_autotune": (_I, [_P, _I, ctypes.POINTER(rbf_tune_report)]),
     "rbf_batch_create": (_I, [ctypes.POINTER(_P), _I, _P]),
@@ -362,6 +367,13 @@ class Solver:
         256) + 1000 x lanes per node (2, 4, 8; 0 for one), or -8 / -16 for one
         cluster of 8 / 16 CTAs."""
         self._ck(self._L.rbf_set_persistent_block(self._h, int(code)))
+
+    def persistent_info(self) -> dict:
+        """Schedule of the last persistent launch: resident (one cell, stencils in shared
+        memory), cluster (CTAs, 0: a grid), threads per block, lanes per node, blocks."""
+        r = rbf_persist_info()
+        self._ck(self._L.rbf_persistent_info(self._h, ctypes.byref(r)))
+        return {f: getattr(r, f) for f, _ in r._fields_}
 
     def set_wait_limit(self, seconds: float):
         """Wall-clock limit of one grid-barrier wait of the persistent ACM driver

@@ -509,7 +509,7 @@ int rbf_build_stencils(rbf_ctx *ctx, int n_l) {
     drop_graph(ctx);
     ctx->weights_ok = false;
     ctx->inited = false;
-    ctx->res_nofit = false;
+    ctx->res_nofit = 0;
     ctx->m_p = 0;
     const int64_t n = ctx->n;
     int G = (int)std::lround(std::cbrt((double)n / 4.0));
@@ -1062,6 +1062,13 @@ int rbf_set_wait_limit(rbf_ctx *ctx, double seconds) {
     return RBF_OK;
 }
 
+int rbf_persistent_info(rbf_ctx *ctx, rbf_persist_info *info) {
+    if (!ctx || !info) return RBF_EINVAL;
+    if (!ctx->persist_info.blocks) return fail(ctx, RBF_EINVAL, "rbf_persistent_info: no persistent launch yet");
+    *info = ctx->persist_info;
+    return RBF_OK;
+}
+
 int rbf_autotune_persistent(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep) {
     if (!ctx) return RBF_EINVAL;
     if (!ctx->inited || ctx->solver != RBF_SOLVER_ACM)
@@ -1370,6 +1377,13 @@ int rbf_pointwise_difference(rbf_ctx *a, rbf_ctx *b, double *delta, double *dv) 
 
 namespace {
 
+// The bit of rbf_ctx::res_nofit for elements of type T and `group` lanes per node: both set
+// how much room a share has for its local nodes.
+template <typename T>
+unsigned res_bit(int group) {
+    return 1u << ((sizeof(T) == 8 ? 4 : 0) + (group == 8 ? 3 : group == 4 ? 2 : group == 2 ? 1 : 0));
+}
+
 // Grid and schedule of a persistent launch over `cs`.
 struct PersistPlan {
     cudaError_t err = cudaSuccess;
@@ -1391,11 +1405,12 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
     if (p.err != cudaSuccess) return p;
     // One cell whose shares fit runs resident, unless one lane per node was asked for (which
     // keeps the summation order of the multi-launch kernels).
-    if (cs.size() == 1 && !x->res_nofit && (!x->persist_block || x->persist_group > 1)) {
+    if (cs.size() == 1 && (!x->persist_block || x->persist_group > 1)) {
         p.group = x->persist_group;
         if (!x->persist_block) resident_auto(x->n / (double)sms, sizeof(T) == 8, &p.block, &p.group);
         else p.block = std::min<int>(sizeof(T) == 4 ? 1024 : 512, std::max<int>(x->persist_block, 256));
-        p.resident = acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, sms, optin - 2048, &p.res);
+        p.resident = !(x->res_nofit & res_bit<T>(p.group)) &&
+                     acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, sms, optin - 2048, &p.res);
         if (p.resident) {
             p.nblocks = p.res.nblocks;
             return p;
@@ -1488,6 +1503,7 @@ int persistent_solve_T(std::vector<rbf_ctx *> &cs, cudaStream_t st, const rbf_so
     else if (pl.csize) CK(acm_launch_persistent_cluster<T>(d_desc, ctl, pl.csize, cp, st));
     else CK(acm_launch_persistent<T>(d_desc, ctl, pl.nblocks, pl.block, pl.group, cp, st));
     CK(cudaEventRecord(ctx->ev1, st));
+    ctx->persist_info = rbf_persist_info{pl.resident, pl.csize, pl.block, pl.group, pl.nblocks};
     std::vector<char> back(o_part - o_bar);
     CK(cudaMemcpyAsync(back.data(), ws + o_bar, back.size(), cudaMemcpyDeviceToHost, st));
     for (rbf_ctx *x : cs) x->launches += 1;
@@ -1508,7 +1524,7 @@ int persistent_solve_T(std::vector<rbf_ctx *> &cs, cudaStream_t st, const rbf_so
         drop_graph(cs[c]);
     }
     if (e == 3) {  // no step was taken: a share's local node set has no room
-        ctx->res_nofit = true;
+        ctx->res_nofit |= res_bit<T>(pl.group);
         return persistent_solve_T<T>(cs, st, o, steps, resid, done, err);
     }
     if (e) {

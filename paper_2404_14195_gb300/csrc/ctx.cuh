@@ -107,7 +107,9 @@ struct rbf_ctx {
     int persist_block = 0;            // threads per block of the persistent ACM driver (0: chosen by size)
     int persist_cluster = 0;          // > 0: run it as one cluster of that many CTAs (8 or 16)
     int persist_group = 1;            // lanes per node of its sweeps (1, 2, 4, 8)
-    bool res_nofit = false;           // a share's local nodes did not fit the resident driver (these stencils)
+    unsigned res_nofit = 0;           // a bit per element size and lanes per node with which a share's local nodes
+                                      // did not fit the resident driver (these stencils)
+    rbf_persist_info persist_info{};  // of its last launch; blocks = 0: none yet
     double persist_ms = 0.0;          // device time of its last launch
     uint64_t wait_ns = 2000000000ull; // wall-clock limit of one grid-barrier wait of that driver
     int gblock = -1;

@@ -1,0 +1,68 @@
+"""Which schedule the persistent ACM driver takes.
+
+A share whose local nodes have no room in shared memory sends the solve to the streaming driver,
+and that answer holds for its element size and lanes per node only.  The cell of 30,306 nodes
+(N_L = 25, 152 SMs) was followed through the shares on the CPU: with one lane per node in FP64 the
+largest share reaches 953 nodes and there is room for 828, with 2 / 4 / 8 lanes 854 / 834 / 817 of
+1296 / 1472 / 1496, in FP32 there is room for 5656 and more.
+"""
+import numpy as np
+import pytest
+
+import synth
+from gpu_common import gpu_or_skip
+
+pytestmark = pytest.mark.gpu
+
+
+def _solver(rbf, case, n_l=25):
+    s = rbf.Solver(0)
+    s.set_case(case)
+    s.build_stencils(n_l)
+    s.compute_weights(solver=rbf.RBF_SOLVER_ACM)
+    return s
+
+
+def test_share_without_room_is_remembered_by_lanes_and_precision():
+    rbf = gpu_or_skip()
+    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=33, seed=8))
+    s.init(precision=rbf.RBF_FP64, v_ref=0.01)
+    with pytest.raises(rbf.RbfError):  # no launch yet
+        s.persistent_info()
+    s.permeability(32)  # the probes of solve()
+    launches, fields = [], []
+    for _ in range(2):
+        s.init(precision=rbf.RBF_FP64, v_ref=0.01)
+        a = s.launch_count()
+        s.solve(4, 1e-300)
+        launches.append(s.launch_count() - a)
+        fields.append(s.get_fields())
+        assert not s.persistent_info()["resident"]
+    assert launches[0] == launches[1] + 1  # the first one found no room, the second did not try again
+    assert np.array_equal(fields[0], fields[1])
+    for lanes in (2, 4, 8):
+        s.set_persistent_block(1000 * lanes + 128)
+        s.solve(4, 1e-300)
+        i = s.persistent_info()
+        assert i["resident"] and i["lanes"] == lanes and i["threads"] == 256, lanes
+    s.close()
+
+
+def test_share_without_room_in_fp64_fits_in_fp32():
+    rbf = gpu_or_skip()
+    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=33, seed=8))
+    for prec, resident in ((rbf.RBF_FP64, 0), (rbf.RBF_FP32, 1), (rbf.RBF_FP32C, 1), (rbf.RBF_FP64, 0)):
+        s.init(precision=prec, v_ref=0.01)
+        s.solve(4, 1e-300)
+        assert s.persistent_info()["resident"] == resident, prec
+    s.close()
+
+
+@pytest.mark.parametrize("n_axis,resident", [(6, 1), (14, 1), (29, 1), (32, 1), (36, 0)])
+def test_resident_up_to_the_capacity(n_axis, resident):
+    rbf = gpu_or_skip()
+    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=n_axis, seed=8))
+    s.init(precision=rbf.RBF_FP64, v_ref=0.01)
+    s.solve(4, 1e-300)
+    assert s.persistent_info()["resident"] == resident
+    s.close()
