@@ -286,8 +286,12 @@ __device__ __forceinline__ T phase_correct(const CellDesc<T> &c, const Sten<T> s
 // PERSIST_SHARED_CELLS cells are copied there too; with more the copies, 250 bytes a cell in
 // every block, take the L1 from the gathers (FP32: 12 cells, 105 steps 51.3 ms with copies, 52.5
 // without; 64 cells, 7.3M nodes 6.55 ms per step with, 5.73 without).
+// The register cap is stated as the warps an SM is to hold: left to itself the compiler takes 96
+// registers in FP64 with several lanes per node (2 blocks an SM instead of 3) and orders the FP32
+// sweeps so that fewer of their loads are in flight (600k nodes, one lane 645 -> 531 us per step; 12
+// cells of 467k 514 -> 421; FP64, 24 cells with four lanes 1.42 -> 1.34 ms).
 template <typename T, bool CP, bool CL, int G, bool SH>
-__global__ void __launch_bounds__(256) k_acm_persistent(const CellDesc<T> *__restrict__ cells_g, PersistCtl ctl) {
+__global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_persistent(const CellDesc<T> *__restrict__ cells_g, PersistCtl ctl) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int nc = ctl.ncells;
     CellDesc<T> *own = reinterpret_cast<CellDesc<T> *>(sm);

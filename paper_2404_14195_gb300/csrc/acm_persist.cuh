@@ -45,6 +45,9 @@ struct PersistCtl {
     unsigned long long *vsq; // resident kernel: 2 slots of max |v|^2
 };
 
+// warps of the streaming kernel's grid on an SM
+template <typename T>
+constexpr int persist_warps() { return sizeof(T) == 4 ? 32 : 24; }
 // cells whose descriptors the streaming kernel copies to shared memory
 constexpr int PERSIST_SHARED_CELLS = 16;
 // shared memory of the streaming kernel: descriptors, residual accumulators, unit counts ahead of each

@@ -66,3 +66,19 @@ def test_resident_up_to_the_capacity(n_axis, resident):
     s.solve(4, 1e-300)
     assert s.persistent_info()["resident"] == resident
     s.close()
+
+
+def test_streaming_blocks_per_sm():
+    """Every lane count has the same warps on an SM: 32 in FP32, 24 in FP64."""
+    rbf = gpu_or_skip()
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=48, seed=8))  # 94k nodes: more units than warps from two lanes
+    for prec, warps in ((rbf.RBF_FP64, 24), (rbf.RBF_FP32, 32)):
+        s.init(precision=prec, v_ref=0.01)
+        for code in (2256, 4256, 4128, 8128):
+            s.set_persistent_block(code)
+            s.solve(2, 1e-300)
+            i = s.persistent_info()
+            assert not i["resident"] and i["blocks"] * i["threads"] == sms * warps * 32, (prec, code)
+    s.close()
