@@ -1416,34 +1416,18 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
             return p;
         }
     }
+    // Streaming: one lane per node unless asked for otherwise.  More lanes only win while a round
+    // of units leaves warps idle (us per step with 256 threads and one lane / 128 and two:
+    // FP32 12 cells 425 / 484, 600k nodes 541 / 597, 113k 181 / 194; FP64 12 cells 1117 / 1317, 24 cells
+    // 1148 / 1150; 15k nodes in 3 cells 108 / 72).
+    p.block = x->persist_block ? x->persist_block : 256;
+    p.group = x->persist_block ? x->persist_group : 1;
     int64_t slices = 0;
     for (const rbf_ctx *y : cs) slices += y->npad / 32;
-    // blocks and the share of the last round's warps that have a unit
-    auto grid = [&](int block, int group, int *nblocks) -> double {
-        int maxb = 0;
-        p.err = acm_persistent_max_blocks<T>(&maxb, block, group, cp, (int)cs.size());
-        const int64_t wpb = block / 32, units = slices * group;
-        *nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(maxb, (units + wpb - 1) / wpb));
-        const double rounds = (double)units / ((double)*nblocks * wpb);
-        return rounds / std::ceil(rounds);
-    };
-    if (x->persist_block) {
-        p.block = x->persist_block;
-        p.group = x->persist_group;
-        grid(p.block, p.group, &p.nblocks);
-        return p;
-    }
-    // One lane per node, unless that leaves the last round of units so empty that two lanes per
-    // node, 8 % slower per unit, finish earlier (485k nodes in 12 cells: 3.1 rounds, 506 us per
-    // step against 484 with two lanes; 600k nodes: 3.9 rounds, 568 against 652)
-    int nb1 = 1, nb2 = 1;
-    const double e1 = grid(256, 1, &nb1);
-    if (p.err != cudaSuccess) return p;
-    const double e2 = grid(128, 2, &nb2);
-    const bool two = 0.92 * e2 > e1;
-    p.block = two ? 128 : 256;
-    p.group = two ? 2 : 1;
-    p.nblocks = two ? nb2 : nb1;
+    int maxb = 0;
+    p.err = acm_persistent_max_blocks<T>(&maxb, p.block, p.group, cp, (int)cs.size());
+    const int64_t wpb = p.block / 32, units = slices * p.group;
+    p.nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(maxb, (units + wpb - 1) / wpb));
     return p;
 }
 

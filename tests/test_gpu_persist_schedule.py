@@ -82,3 +82,27 @@ def test_streaming_blocks_per_sm():
             i = s.persistent_info()
             assert not i["resident"] and i["blocks"] * i["threads"] == sms * warps * 32, (prec, code)
     s.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp32c"])
+def test_batch_default_is_one_lane_per_node(prec):
+    """24 cells, about 12,300 units: 3.4 rounds of an FP64 grid's 3,648 warps, 2.5 of an FP32 grid's
+    4,864.  One lane per node, and the same fields from blocks of 32 threads."""
+    rbf = gpu_or_skip()
+    b = rbf.Batch(0)
+    cells = [synth.jittered_cell(r=0.3, n_axis=25 + i % 3, seed=40 + i) for i in range(24)]
+    for c in cells:
+        b.add_cell(c, 20)
+    b.build(3, 2)
+    p = {"fp64": rbf.RBF_FP64, "fp32": rbf.RBF_FP32, "fp32c": rbf.RBF_FP32C}[prec]
+    got = []
+    for code in (None, 32):
+        if code:
+            b.set_persistent_block(code)
+        b.init(precision=p, v_ref=0.01)
+        assert [r["steps"] for r in b.solve(6, 1e-300, check_every=3)] == [6] * 24
+        i = b.cell(0).persistent_info()
+        assert i["lanes"] == 1 and i["threads"] == (code or 256) and not i["resident"]
+        got.append([b.cell(j).get_fields() for j in range(24)])
+    for x, y in zip(*got):
+        assert np.abs(x).max() > 0 and np.array_equal(x, y)
