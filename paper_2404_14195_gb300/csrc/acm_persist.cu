@@ -282,10 +282,8 @@ __device__ __forceinline__ T phase_correct(const CellDesc<T> &c, const Sten<T> s
 // synchronised by the cluster's hardware barrier.  Every block of a cluster takes the
 // same branches at every barrier (the done flags change only before a barrier and
 // the cluster barrier cannot time out), so none is left waiting.  Dynamic shared
-// memory: residual sums, unit counts and flags of the cells.  SH: the descriptors of up to
-// PERSIST_SHARED_CELLS cells are copied there too; with more the copies, 250 bytes a cell in
-// every block, take the L1 from the gathers (FP32: 12 cells, 105 steps 51.3 ms with copies, 52.5
-// without; 64 cells, 7.3M nodes 6.55 ms per step with, 5.73 without).
+// memory: residual sums, unit counts and flags of the cells; with SH (persist_shared) also
+// copies of the descriptors.
 // The register cap is stated as the warps an SM is to hold: left to itself the compiler takes 96
 // registers in FP64 with several lanes per node (2 blocks an SM instead of 3) and orders the FP32
 // sweeps so that fewer of their loads are in flight (600k nodes, one lane 645 -> 531 us per step; 12
@@ -1002,7 +1000,6 @@ cudaError_t launch_cluster_T(const CellDesc<T> *cells_dev, const PersistCtl &ctl
                              int *max_clusters) {
     auto kern = k_acm_persistent<T, CP, true, 1, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
@@ -1026,11 +1023,11 @@ cudaError_t launch_cluster_T(const CellDesc<T> *cells_dev, const PersistCtl &ctl
 template <typename T>
 cudaError_t acm_launch_persistent(const CellDesc<T> *cells_dev, const PersistCtl &ctl, int nblocks, int block,
                                   int group, bool cp, cudaStream_t st) {
-    const void *fn = grid_kernel<T>(group, cp, ctl.ncells <= PERSIST_SHARED_CELLS);
-    if (!persist_block_ok(block) || nblocks < 1 || !fn) return cudaErrorInvalidValue;
-    const size_t smem = persist_head_bytes<T>(ctl.ncells);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (!persist_block_ok(block) || nblocks < 1) return cudaErrorInvalidValue;
+    const bool sh = persist_shared<T>(ctl.ncells, block);
+    const void *fn = grid_kernel<T>(group, cp, sh);
+    if (!fn) return cudaErrorInvalidValue;
+    const size_t smem = persist_head_bytes<T>(ctl.ncells, sh);
     void *args[] = {(void *)&cells_dev, (void *)&ctl};
     return cudaLaunchCooperativeKernel(fn, dim3(nblocks), dim3(block), args, smem, st);
 }
@@ -1039,7 +1036,7 @@ template <typename T>
 cudaError_t acm_launch_persistent_cluster(const CellDesc<T> *cells_dev, const PersistCtl &ctl, int csize, bool cp,
                                           cudaStream_t st) {
     if (csize != 8 && csize != 16) return cudaErrorInvalidValue;
-    const size_t smem = persist_head_bytes<T>(ctl.ncells);
+    const size_t smem = persist_head_bytes<T>(ctl.ncells, false);
     return cp ? launch_cluster_T<T, true>(cells_dev, ctl, csize, smem, st, nullptr)
               : launch_cluster_T<T, false>(cells_dev, ctl, csize, smem, st, nullptr);
 }
@@ -1061,13 +1058,14 @@ cudaError_t acm_persistent_cluster_ok(int csize, bool cp, size_t smem, bool *ok)
 
 template <typename T>
 cudaError_t acm_persistent_max_blocks(int *blocks, int block, int group, bool cp, int ncells) {
-    const size_t smem = persist_head_bytes<T>(ncells);
-    const void *fn = grid_kernel<T>(group, cp, ncells <= PERSIST_SHARED_CELLS);
-    if (!persist_block_ok(block) || !fn) return cudaErrorInvalidValue;
+    if (!persist_block_ok(block)) return cudaErrorInvalidValue;
+    const bool sh = persist_shared<T>(ncells, block);
+    const size_t smem = persist_head_bytes<T>(ncells, sh);
+    const void *fn = grid_kernel<T>(group, cp, sh);
+    if (!fn) return cudaErrorInvalidValue;
     int dev = 0, sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, block, smem);
     *blocks = sms * per;
     return e;

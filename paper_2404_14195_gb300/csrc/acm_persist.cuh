@@ -48,13 +48,21 @@ struct PersistCtl {
 // warps of the streaming kernel's grid on an SM
 template <typename T>
 constexpr int persist_warps() { return sizeof(T) == 4 ? 32 : 24; }
-// cells whose descriptors the streaming kernel copies to shared memory
-constexpr int PERSIST_SHARED_CELLS = 16;
-// shared memory of the streaming kernel: descriptors, residual accumulators, unit counts ahead of each
-// cell, flags
+// Whether its blocks of `block` threads copy the descriptors to shared memory: while an SM's copies
+// take 64 kB at most.  A field's address is then a shared-memory load, but the copies take
+// room from the L1, and from the blocks themselves past that.  Time with copies over time
+// without, FP32 (FP64 within 2 %), by cells / threads (kB of copies per SM):
+//   1 / 256 (1) 0.96, 12 / 256 (14) 0.96, 24 / 256 (28) 0.95, 24 / 128 (55) 0.96, 64 / 256 (74) 0.98 to 1.01,
+//   40 / 128 (92) 0.96, 12 / 32 (111) 1.01, 64 / 128 (147) 1.15 to 1.21, 40 / 64 (184) 1.91
 template <typename T>
-__host__ __device__ constexpr int64_t persist_head_bytes(int ncells) {
-    return ((ncells <= PERSIST_SHARED_CELLS ? ncells : 0) * (int64_t)sizeof(CellDesc<T>) + (ncells + 1) * 16ll + ncells * 16ll + ncells * 4ll + 15) & ~15ll;
+constexpr bool persist_shared(int ncells, int block) {
+    return (int64_t)ncells * (int64_t)sizeof(CellDesc<T>) * (persist_warps<T>() * 32 / block) <= 65536;
+}
+// its shared memory: descriptors, residual accumulators, unit counts ahead of each cell, flags; below
+// the 48 kB that a launch may ask for without further ado
+template <typename T>
+constexpr int64_t persist_head_bytes(int ncells, bool shared) {
+    return ((shared ? ncells : 0) * (int64_t)sizeof(CellDesc<T>) + (ncells + 1) * 16ll + ncells * 16ll + ncells * 4ll + 15) & ~15ll;
 }
 // Shares of the resident kernel (one cell, every block's stencils in shared memory):
 // largest number of units and wall units per block, local nodes there is room for,
@@ -77,7 +85,7 @@ cudaError_t acm_launch_resident(const CellDesc<T> &cell, const PersistCtl &ctl, 
 template <typename T>
 cudaError_t acm_launch_persistent(const CellDesc<T> *cells_dev, const PersistCtl &ctl, int nblocks, int block,
                                   int group, bool cp, cudaStream_t st);
-// co-resident blocks of the kernel with `smem` bytes of dynamic shared memory each
+// co-resident blocks of the kernel over `ncells` cells
 template <typename T>
 cudaError_t acm_persistent_max_blocks(int *blocks, int block, int group, bool cp, int ncells);
 // the same kernel as one thread-block cluster of csize (8 or 16) CTAs of 256

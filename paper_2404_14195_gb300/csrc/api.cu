@@ -1001,8 +1001,8 @@ int tune_persistent(std::vector<rbf_ctx *> &cs, int trial_steps, rbf_tune_report
     for (int c : {16, 8}) {
         bool ok = false;
         const int nc = (int)cs.size();
-        if (is_f32(ctx)) CK(acm_persistent_cluster_ok<float>(c, ctx->prec == RBF_FP32C, (size_t)persist_head_bytes<float>(nc), &ok));
-        else CK(acm_persistent_cluster_ok<double>(c, false, (size_t)persist_head_bytes<double>(nc), &ok));
+        if (is_f32(ctx)) CK(acm_persistent_cluster_ok<float>(c, ctx->prec == RBF_FP32C, (size_t)persist_head_bytes<float>(nc, false), &ok));
+        else CK(acm_persistent_cluster_ok<double>(c, false, (size_t)persist_head_bytes<double>(nc, false), &ok));
         if (ok) cands.push_back(-c);
     }
     rbf_tune_report r;

@@ -106,3 +106,22 @@ def test_batch_default_is_one_lane_per_node(prec):
         got.append([b.cell(j).get_fields() for j in range(24)])
     for x, y in zip(*got):
         assert np.abs(x).max() > 0 and np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_descriptor_copies_change_nothing(prec):
+    """40 cells: blocks of 256 threads hold copies of the descriptors in shared memory (46 kB per SM), blocks of 64
+    and 32 read them from global memory (150 kB and more)."""
+    rbf = gpu_or_skip()
+    b = rbf.Batch(0)
+    for i in range(40):
+        b.add_cell(synth.jittered_cell(r=0.3, n_axis=7 + i % 2, seed=60 + i), 20)
+    b.build(3, 2)
+    got = []
+    for code in (256, 64, 32):
+        b.init(precision=rbf.RBF_FP64 if prec == "fp64" else rbf.RBF_FP32, v_ref=0.01)
+        b.set_persistent_block(code)
+        assert [r["steps"] for r in b.solve(20, 1e-300, check_every=7)] == [20] * 40
+        got.append([b.cell(j).get_fields() for j in range(40)])
+    for j in range(40):
+        assert np.abs(got[0][j]).max() > 0 and all(np.array_equal(g[j], got[0][j]) for g in got[1:]), j
