@@ -230,11 +230,6 @@ __global__ void k_acm_vmax(AcmArgs<T> a, int slot) {
     if ((threadIdx.x & 31) == 0 && sp > 0.0) atomicMax(a.vmax + slot, (unsigned long long)__double_as_longlong(sp));
 }
 
-// Lanes per node of the wall sweep: wall nodes are few (60k of 600k) and one lane's 25 dependent
-// gathers are the sweep's time, so four lanes share them at every schedule (FP32 step of 600k
-// nodes 586 -> 571 us; one lane per wall node 18.8 us of each of its three wall sweeps).
-constexpr int WALL_LANES = 4;
-
 // Iteration g of the run (counted over all steps) writes max |v| into slot g % 2;
 // the pressure sweep of iteration g reads slot (g + 1) % 2 (the previous
 // iteration's) and clears slot g % 2 for its own correction sweep.  The grids

@@ -71,6 +71,13 @@ inline int acm_code_auto(int64_t n, int sms, bool fp64) {
     return n <= sms * four ? 4128 : n <= sms * two ? 2128 : 256;
 }
 
+// Lanes per node of the wall sweep: wall nodes are few (102k of 600k) and one lane's n_l - 1
+// dependent gathers are the sweep's time, so four lanes share them at every schedule (FP32 step of
+// 600k nodes, N_L = 40: 586 -> 571 us; one lane per wall node 18.8 us of each of its three wall
+// sweeps).  The streaming persistent driver has the same (FP32 step of 6 cells, 113k nodes: 181 ->
+// 159 us, 52k nodes 94 -> 81; FP64 112k nodes 244 -> 235, 12 cells of 467k 1120 -> 1147).
+constexpr int WALL_LANES = 4;
+
 template <typename T>
 cudaError_t acm_launch_step(const AcmArgs<T> &a, int n_p, int parity, cudaStream_t st, int64_t *launches,
                             LaunchRecorder *rec = nullptr, int code = 256);

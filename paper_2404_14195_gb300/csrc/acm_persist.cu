@@ -9,7 +9,8 @@
 // cell, |v - v_prev|^2 and |v|^2 in FP64, block 0 turns them into residuals and sets
 // the cell's done flag; converged cells drop out of the loop while the others
 // continue.  The arithmetic of each phase is that of the multi-launch kernels in
-// acm.cu (for G = 1 in the same order).
+// acm.cu, in the same order for the same lanes per node (wall nodes have WALL_LANES in both),
+// except in the resident kernel.
 //
 // What bounds it, and the layout that follows: a step of a small cell is ten phases
 // of a few hundred nanoseconds of work each, so the chain barrier -> descriptor ->
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
         for (int c = threadIdx.x; c < nc; c += blockDim.x) {
             done[c] = 0;
             pre[c + 1] = ((cells_g[c].n + 31) >> 5) * G;
-            wpre[c + 1] = ((cells_g[c].nb + 31) >> 5) * G;
+            wpre[c + 1] = ((cells_g[c].nb + 31) >> 5) * WALL_LANES;
         }
     }
     __syncthreads();
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
             while (k >= wpre[c + 1]) ++c;
             if (done[c]) continue;
             const int64_t un = k - wpre[c];
-            f(cells[c], un / G, (int)(un % G));
+            f(cells[c], un / WALL_LANES, (int)(un % WALL_LANES));
         }
     };
     auto sten = [&](const CellDesc<T> &d, int64_t ls, int nl) {
@@ -416,9 +417,9 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
             });
             if (!barrier()) { broke = true; break; }
             wall_units([&](const CellDesc<T> &d, int64_t ls, int sub) {
-                const int nl = sub * NU + nl0;
-                phase_wall<T, CP, G>(d, Sten<T>{d.wn + ((ls * d.n_l) << 5) + nl, d.idxb + ((ls * d.n_l) << 5) + nl},
-                                     (ls << 5) + nl, g);
+                const int nl = sub * (32 / WALL_LANES) + lane / WALL_LANES;
+                phase_wall<T, CP, WALL_LANES>(d, Sten<T>{d.wn + ((ls * d.n_l) << 5) + nl, d.idxb + ((ls * d.n_l) << 5) + nl},
+                                              (ls << 5) + nl, lane % WALL_LANES);
             });
             if (!barrier()) { broke = true; break; }
             // max |v| of each cell: the largest |v|^2 of this warp's units, one root and one

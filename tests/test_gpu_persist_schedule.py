@@ -125,3 +125,22 @@ def test_descriptor_copies_change_nothing(prec):
         got.append([b.cell(j).get_fields() for j in range(40)])
     for j in range(40):
         assert np.abs(got[0][j]).max() > 0 and all(np.array_equal(g[j], got[0][j]) for g in got[1:]), j
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_one_lane_solve_equals_the_step_kernels(prec):
+    """Code 256 of both: the same sums in the same order, so the same bits."""
+    rbf = gpu_or_skip()
+    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=14, seed=5))
+    got = []
+    for solve in (0, 1):
+        s.init(precision=rbf.RBF_FP64 if prec == "fp64" else rbf.RBF_FP32, v_ref=0.01)
+        if solve:
+            s.set_persistent_block(256)
+            s.solve(40, 1e-300)
+        else:
+            s.set_kernel_variant(256)
+            s.step(40)
+        got.append(s.get_fields())
+    assert np.abs(got[0]).max() > 0 and np.array_equal(*got)
+    s.close()
