@@ -301,7 +301,9 @@ int rbf_autotune(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep);
  * by a software grid barrier) and, where the device can place them, one
  * thread-block cluster of 16 or 8 CTAs synchronised by the hardware cluster
  * barrier (codes -16, -8), over trial_steps steps each, CUDA events around the
- * launch, and keep the fastest for this context's later rbf_solve calls.  Fields
+ * launch, and keep the fastest for this context's later rbf_solve calls.  The
+ * schedule chosen by size (code 0) is timed too unless one of the others is the
+ * same launch.  Fields
  * and step parity are saved before and restored after the trials.  ACM contexts
  * only; 2 <= trial_steps <= 20000.  rep->code[c] is the code of candidate c. */
 int rbf_autotune_persistent(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep);
@@ -314,8 +316,10 @@ int rbf_autotune_persistent(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep)
  *                    With G > 1 a single cell whose stencils fit the SMs' shared
  *                    memory runs resident there, one block of at least 256
  *                    threads per SM;
- *   -8, -16          one cluster of 8 / 16 CTAs of 256 threads, G = 1.
- * Until a code is set the schedule is chosen by the size of the cells.
+ *   -8, -16          one cluster of 8 / 16 CTAs of 256 threads, G = 1;
+ *   0                chosen by the size of the cells, as until a code is set: one cell
+ *                    whose stencils fit resident with 1, 2 or 4 lanes per node and 256
+ *                    or 512 threads, everything else as 256.
  * A batch launches with its first cell's setting.  With G = 1 the schedule
  * changes only the order of the FP64 residual partial sums; G > 1 also changes
  * the order of the stencil sums (rounding only). */

@@ -364,8 +364,8 @@ class Solver:
 
     def set_persistent_block(self, code: int):
         """Persistent ACM driver schedule code: threads per block (32, 64, 128,
-        256) + 1000 x lanes per node (2, 4, 8; 0 for one), or -8 / -16 for one
-        cluster of 8 / 16 CTAs."""
+        256) + 1000 x lanes per node (2, 4, 8; 0 for one), -8 / -16 for one
+        cluster of 8 / 16 CTAs, or 0 for the schedule by size (the default)."""
         self._ck(self._L.rbf_set_persistent_block(self._h, int(code)))
 
     def persistent_info(self) -> dict:
@@ -381,9 +381,10 @@ class Solver:
         self._ck(self._L.rbf_set_wait_limit(self._h, float(seconds)))
 
     def autotune_persistent(self, trial_steps: int = 200):
-        """ACM: time the persistent driver's block sizes on this case and keep the
+        """ACM: time the persistent driver's schedules on this case and keep the
         fastest for solve(); the state is restored afterwards.  Returns
-        {threads per block: ms_per_step}, chosen."""
+        {code: ms_per_step}, chosen (codes as at set_persistent_block; 0 only where
+        no other code is the schedule by size)."""
         r = rbf_tune_report()
         self._ck(self._L.rbf_autotune_persistent(self._h, int(trial_steps), ctypes.byref(r)))
         return {r.code[i]: r.ms_per_step[i] for i in range(r.n_candidates)}, r.chosen

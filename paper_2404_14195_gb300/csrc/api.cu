@@ -963,11 +963,65 @@ int rbf_autotune(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep) {
 }  // extern "C"
 
 namespace {
+// The bit of rbf_ctx::res_nofit for elements of type T and `group` lanes per node: both set
+// how much room a share has for its local nodes.
+template <typename T>
+unsigned res_bit(int group) {
+    return 1u << ((sizeof(T) == 8 ? 4 : 0) + (group == 8 ? 3 : group == 4 ? 2 : group == 2 ? 1 : 0));
+}
+
+// Grid and schedule of a persistent launch over `cs`.
+struct PersistPlan {
+    cudaError_t err = cudaSuccess;
+    int csize = 0, nblocks = 1, block = 256, group = 1;
+    bool resident = false;
+    ResPlan res{};
+};
+template <typename T>
+PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
+    PersistPlan p;
+    const rbf_ctx *x = cs[0];
+    if (x->persist_cluster) {
+        p.csize = p.nblocks = x->persist_cluster;
+        return p;
+    }
+    int sms = 0, optin = 0;
+    p.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, x->device);
+    if (p.err == cudaSuccess) p.err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, x->device);
+    if (p.err != cudaSuccess) return p;
+    // One cell whose shares fit runs resident, unless one lane per node was asked for (which
+    // keeps the summation order of the multi-launch kernels).
+    if (cs.size() == 1 && (!x->persist_block || x->persist_group > 1)) {
+        p.group = x->persist_group;
+        if (!x->persist_block) resident_auto(x->n / (double)sms, sizeof(T) == 8, &p.block, &p.group);
+        else p.block = std::min<int>(sizeof(T) == 4 ? 1024 : 512, std::max<int>(x->persist_block, 256));
+        p.resident = !(x->res_nofit & res_bit<T>(p.group)) &&
+                     acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, sms, optin - 2048, &p.res);
+        if (p.resident) {
+            p.nblocks = p.res.nblocks;
+            return p;
+        }
+    }
+    // Streaming: one lane per node unless asked for otherwise.  More lanes only win while a round
+    // of units leaves warps idle (us per step with 256 threads and one lane / 128 and two:
+    // FP32 12 cells 425 / 484, 600k nodes 541 / 597, 113k 181 / 194; FP64 12 cells 1117 / 1317, 24 cells
+    // 1148 / 1150; 15k nodes in 3 cells 108 / 72).
+    p.block = x->persist_block ? x->persist_block : 256;
+    p.group = x->persist_block ? x->persist_group : 1;
+    int64_t slices = 0;
+    for (const rbf_ctx *y : cs) slices += y->npad / 32;
+    int maxb = 0;
+    p.err = acm_persistent_max_blocks<T>(&maxb, p.block, p.group, cp, (int)cs.size());
+    const int64_t wpb = p.block / 32, units = slices * p.group;
+    p.nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(maxb, (units + wpb - 1) / wpb));
+    return p;
+}
+
 // schedule code of the persistent driver: block (32 .. 256) + 1000 group for a grid
 // with `group` lanes per node (group 1: the code is the block size), -8 / -16 for a
-// cluster; false for anything else
+// cluster, 0 by size; false for anything else
 bool persist_code_ok(int code) {
-    if (code == -8 || code == -16) return true;
+    if (code == 0 || code == -8 || code == -16) return true;
     const int block = code % 1000, group = code / 1000;
     return (block == 32 || block == 64 || block == 128 || block == 256) &&
            (group == 0 || group == 2 || group == 4 || group == 8);
@@ -982,8 +1036,9 @@ void set_persist_code(rbf_ctx *x, int code) {
     x->persist_group = code / 1000 ? code / 1000 : 1;
 }
 
-// Time the persistent driver over `cs` for every block size and keep the fastest
-// in every cell; the cells' fields and parities are restored after each trial.
+// Time the persistent driver over `cs` for every schedule and keep the fastest
+// in every cell; the cells' fields and parities are restored after each trial.  The
+// schedule by size (code 0) is a candidate of its own where no other code launches the same.
 int tune_persistent(std::vector<rbf_ctx *> &cs, int trial_steps, rbf_tune_report *rep, std::string &err) {
     rbf_ctx *ctx = cs[0];
     std::vector<StateCopy> sc(cs.size());
@@ -1005,6 +1060,20 @@ int tune_persistent(std::vector<rbf_ctx *> &cs, int trial_steps, rbf_tune_report
         else CK(acm_persistent_cluster_ok<double>(c, false, (size_t)persist_head_bytes<double>(nc, false), &ok));
         if (ok) cands.push_back(-c);
     }
+    auto plan = [&](int code) {
+        for (rbf_ctx *x : cs) set_persist_code(x, code);
+        return is_f32(ctx) ? persist_plan<float>(cs, ctx->prec == RBF_FP32C) : persist_plan<double>(cs, false);
+    };
+    const PersistPlan by_size = plan(0);
+    CK(by_size.err);
+    bool covered = false;
+    for (int code : cands) {
+        const PersistPlan p = plan(code);
+        CK(p.err);
+        covered |= p.csize == by_size.csize && p.resident == by_size.resident && p.block == by_size.block &&
+                   p.group == by_size.group && p.nblocks == by_size.nblocks;
+    }
+    if (!covered) cands.insert(cands.begin(), 0);
     rbf_tune_report r;
     std::memset(&r, 0, sizeof(r));
     double best = 1e300;
@@ -1049,7 +1118,7 @@ int rbf_set_persistent_block(rbf_ctx *ctx, int code) {
     if (!ctx) return RBF_EINVAL;
     if (!persist_code_ok(code))
         return fail(ctx, RBF_EINVAL, "rbf_set_persistent_block: code = block (32, 64, 128, 256) + 1000 x lanes per "
-                                     "node (2, 4, 8; 0 for 1), or -8 / -16");
+                                     "node (2, 4, 8; 0 for 1), -8 / -16, or 0 (by size)");
     set_persist_code(ctx, code);
     return RBF_OK;
 }
@@ -1376,60 +1445,6 @@ int rbf_pointwise_difference(rbf_ctx *a, rbf_ctx *b, double *delta, double *dv) 
 }  // extern "C"
 
 namespace {
-
-// The bit of rbf_ctx::res_nofit for elements of type T and `group` lanes per node: both set
-// how much room a share has for its local nodes.
-template <typename T>
-unsigned res_bit(int group) {
-    return 1u << ((sizeof(T) == 8 ? 4 : 0) + (group == 8 ? 3 : group == 4 ? 2 : group == 2 ? 1 : 0));
-}
-
-// Grid and schedule of a persistent launch over `cs`.
-struct PersistPlan {
-    cudaError_t err = cudaSuccess;
-    int csize = 0, nblocks = 1, block = 256, group = 1;
-    bool resident = false;
-    ResPlan res{};
-};
-template <typename T>
-PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
-    PersistPlan p;
-    const rbf_ctx *x = cs[0];
-    if (x->persist_cluster) {
-        p.csize = p.nblocks = x->persist_cluster;
-        return p;
-    }
-    int sms = 0, optin = 0;
-    p.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, x->device);
-    if (p.err == cudaSuccess) p.err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, x->device);
-    if (p.err != cudaSuccess) return p;
-    // One cell whose shares fit runs resident, unless one lane per node was asked for (which
-    // keeps the summation order of the multi-launch kernels).
-    if (cs.size() == 1 && (!x->persist_block || x->persist_group > 1)) {
-        p.group = x->persist_group;
-        if (!x->persist_block) resident_auto(x->n / (double)sms, sizeof(T) == 8, &p.block, &p.group);
-        else p.block = std::min<int>(sizeof(T) == 4 ? 1024 : 512, std::max<int>(x->persist_block, 256));
-        p.resident = !(x->res_nofit & res_bit<T>(p.group)) &&
-                     acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, sms, optin - 2048, &p.res);
-        if (p.resident) {
-            p.nblocks = p.res.nblocks;
-            return p;
-        }
-    }
-    // Streaming: one lane per node unless asked for otherwise.  More lanes only win while a round
-    // of units leaves warps idle (us per step with 256 threads and one lane / 128 and two:
-    // FP32 12 cells 425 / 484, 600k nodes 541 / 597, 113k 181 / 194; FP64 12 cells 1117 / 1317, 24 cells
-    // 1148 / 1150; 15k nodes in 3 cells 108 / 72).
-    p.block = x->persist_block ? x->persist_block : 256;
-    p.group = x->persist_block ? x->persist_group : 1;
-    int64_t slices = 0;
-    for (const rbf_ctx *y : cs) slices += y->npad / 32;
-    int maxb = 0;
-    p.err = acm_persistent_max_blocks<T>(&maxb, p.block, p.group, cp, (int)cs.size());
-    const int64_t wpb = p.block / 32, units = slices * p.group;
-    p.nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(maxb, (units + wpb - 1) / wpb));
-    return p;
-}
 
 // Steady ACM solve of one or more initialised contexts (same device, stream,
 // precision and n_p) in one persistent cooperative launch.  Per cell: steps taken,

@@ -144,3 +144,42 @@ def test_one_lane_solve_equals_the_step_kernels(prec):
         got.append(s.get_fields())
     assert np.abs(got[0]).max() > 0 and np.array_equal(*got)
     s.close()
+
+
+@pytest.mark.parametrize("prec,n_axis,lanes,threads", [("fp32", 34, 1, 512), ("fp32c", 34, 1, 512), ("fp64", 24, 2, 512)])
+def test_tuner_times_the_schedule_by_size(prec, n_axis, lanes, threads):
+    """Where no code names the schedule by size (512 threads, one lane resident) it is a candidate, code 0, so
+    that tuning cannot lose it; setting 0 returns to it."""
+    rbf = gpu_or_skip()
+    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=n_axis, seed=8))
+    s.init(precision={"fp64": rbf.RBF_FP64, "fp32": rbf.RBF_FP32, "fp32c": rbf.RBF_FP32C}[prec], v_ref=0.01)
+    want = dict(resident=1, cluster=0, threads=threads, lanes=lanes)
+    s.solve(2, 1e-300)
+    i = s.persistent_info()
+    assert {k: i[k] for k in want} == want
+    before = s.get_fields()
+    times, chosen = s.autotune_persistent(100)
+    assert np.array_equal(s.get_fields(), before)
+    assert 0 in times and times[chosen] == min(times.values()) <= times[0]
+    s.set_persistent_block(256)
+    s.solve(2, 1e-300)
+    assert not s.persistent_info()["resident"]
+    s.set_persistent_block(0)
+    s.solve(2, 1e-300)
+    i = s.persistent_info()
+    assert {k: i[k] for k in want} == want
+    s.close()
+
+
+def test_tuner_names_the_schedule_by_size_once():
+    rbf = gpu_or_skip()
+    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=14, seed=5))  # by size: 256 threads, four lanes, as 4256
+    s.init(precision=rbf.RBF_FP64, v_ref=0.01)
+    assert 0 not in s.autotune_persistent(20)[0]
+    s.close()
+    b = rbf.Batch(0)
+    for i in range(2):
+        b.add_cell(synth.jittered_cell(r=0.3, n_axis=12, seed=70 + i), 20)
+    b.build(3, 2)
+    b.init(precision=rbf.RBF_FP32, v_ref=0.01)
+    assert 0 not in b.autotune(20)[0]  # as 256
