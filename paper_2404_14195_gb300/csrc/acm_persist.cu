@@ -1098,7 +1098,10 @@ cudaError_t acm_launch_resident(const CellDesc<T> &cell, const PersistCtl &ctl, 
                                 bool cp, cudaStream_t st) {
     const void *fn = cp ? resident_kernel<T, true>(group) : resident_kernel<T, false>(group);
     if (block < 32 || block % 32 || block > (sizeof(T) == 4 ? 1024 : 512) || !fn) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.smem);
+    // the kernel's limit is one for all threads of the program: always the same value
+    int room = 0;
+    cudaError_t e = resident_room(&room);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
     if (e != cudaSuccess) return e;
     void *args[] = {(void *)&cell, (void *)&ctl, (void *)&pl};
     return cudaLaunchCooperativeKernel(fn, dim3(pl.nblocks), dim3(block), args, (size_t)pl.smem, st);

@@ -985,9 +985,9 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
         p.csize = p.nblocks = x->persist_cluster;
         return p;
     }
-    int sms = 0, optin = 0;
+    int sms = 0, room = 0;
     p.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, x->device);
-    if (p.err == cudaSuccess) p.err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, x->device);
+    if (p.err == cudaSuccess) p.err = resident_room(&room);
     if (p.err != cudaSuccess) return p;
     // One cell whose shares fit runs resident, unless one lane per node was asked for (which
     // keeps the summation order of the multi-launch kernels).
@@ -996,7 +996,7 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
         if (!x->persist_block) resident_auto(x->n / (double)sms, sizeof(T) == 8, &p.block, &p.group);
         else p.block = std::min<int>(sizeof(T) == 4 ? 1024 : 512, std::max<int>(x->persist_block, 256));
         p.resident = !(x->res_nofit & res_bit<T>(p.group)) &&
-                     acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, sms, optin - 2048, &p.res);
+                     acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, sms, room, &p.res);
         if (p.resident) {
             p.nblocks = p.res.nblocks;
             return p;

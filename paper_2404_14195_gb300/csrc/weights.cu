@@ -908,9 +908,16 @@ __global__ void __launch_bounds__(WT) k_weights(WSet S, int64_t ntot, const int3
     }
 }
 
+// A kernel's shared-memory limit is one for all threads of the program, so it is always set to
+// the same value, the largest system's: with each launch's own, another thread's smaller one
+// in between made the launch fail.
+cudaError_t set_limit(const void *kern, size_t bytes) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 cudaError_t launch_set(const WSet &S, int64_t ntot, int max_n_l, int k, int np, int n_ops, int32_t *list, cudaStream_t st) {
     const size_t smem = wlayout(max_n_l, np, n_ops).total * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = set_limit((const void *)k_weights, wlayout(RBF_MAX_NL, RBF_MAX_NP, RBF_MAX_OPS).total * sizeof(double));
     if (e != cudaSuccess) return e;
     if (k > 5) {
         k_weights<<<(unsigned)ntot, WT, smem, st>>>(S, ntot, nullptr);
@@ -920,7 +927,7 @@ cudaError_t launch_set(const WSet &S, int64_t ntot, int max_n_l, int k, int np, 
     // the smallest register tile that holds the system
     const int ns = max_n_l + np;
     auto *kern = ns <= 48 ? k_weights_fast<3, 6> : ns <= 64 ? k_weights_fast<4, 8> : k_weights_fast<7, 13>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
+    e = set_limit((const void *)kern, flayout(RBF_MAX_NL, RBF_MAX_NP, RBF_MAX_OPS).total);
     if (e == cudaSuccess) e = cudaMemsetAsync(list, 0, sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)ntot, WT, fsmem, st>>>(S, list);
