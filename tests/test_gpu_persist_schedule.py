@@ -183,3 +183,35 @@ def test_tuner_names_the_schedule_by_size_once():
     b.build(3, 2)
     b.init(precision=rbf.RBF_FP32, v_ref=0.01)
     assert 0 not in b.autotune(20)[0]  # as 256
+
+
+@pytest.mark.parametrize("prec,big", [("fp64", 1.7e308), ("fp32", 3.3e38)])
+def test_wall_pressure_beyond_the_range(prec, big):
+    """One fluid node's pressure near the largest value: a wall sum that overflows gives the same infinity in
+    the resident driver as in the streaming one, and where it does not the same quotient (each sum has one
+    term that counts: 4 eps)."""
+    rbf = gpu_or_skip()
+    case = synth.jittered_cell(r=0.35, n_axis=14, seed=5)
+    s = _solver(rbf, case)
+    wall = case["type"] == 1
+    d = np.abs(np.linalg.norm(case["xyz"] - 0.5, axis=1) - 0.35)
+    d[wall] = 1.0
+    start = np.zeros((case.n, 4))
+    start[d.argmin(), 3] = big
+    p = []
+    for code in (256, 4128):
+        s.init(precision=rbf.RBF_FP64 if prec == "fp64" else rbf.RBF_FP32, v_ref=0.01, n_p=1)
+        s.set_persistent_block(code)
+        s.set_fields(start)
+        with pytest.raises(rbf.RbfError) as ei:
+            s.solve(1, 1e-300)
+        assert ei.value.code == rbf.RBF_EDIVERGED
+        assert s.persistent_info()["resident"] == (code == 4128)
+        p.append(s.get_fields()[wall, 3])
+    inf = np.isinf(p[0])
+    assert inf.any() and (~inf & (np.abs(p[0]) > 1e-3 * big)).any() and not np.isnan(p[0]).any()
+    assert np.array_equal(p[0][inf], p[1][inf])
+    eps = 2.0 ** (-52 if prec == "fp64" else -23)
+    x, y = p[0][~inf], p[1][~inf]
+    assert (np.abs(x - y) <= 4 * eps * np.abs(x) + 1e-30 * big).all()
+    s.close()
