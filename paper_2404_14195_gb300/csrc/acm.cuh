@@ -74,8 +74,8 @@ inline int acm_code_auto(int64_t n, int sms, bool fp64) {
 // Lanes per node of the wall sweep: wall nodes are few (102k of 600k) and one lane's n_l - 1
 // dependent gathers are the sweep's time, so four lanes share them at every schedule (FP32 step of
 // 600k nodes, N_L = 40: 586 -> 571 us; one lane per wall node 18.8 us of each of its three wall
-// sweeps).  The streaming persistent driver has the same (FP32 step of 6 cells, 113k nodes: 181 ->
-// 159 us, 52k nodes 94 -> 81; FP64 112k nodes 244 -> 235, 12 cells of 467k 1120 -> 1147).
+// sweeps).  The streaming persistent driver sums in the same order (a step of 6 FP32 cells, 113k
+// nodes: 181 -> 168 us, 52k nodes 94 -> 87; FP64 112k nodes 244 -> 235).
 constexpr int WALL_LANES = 4;
 
 template <typename T>

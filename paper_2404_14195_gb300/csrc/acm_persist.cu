@@ -62,10 +62,10 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
 // Arrive and wait until every block has arrived for this barrier: bar[0] counts arrivals
 // (it only grows; `target` is its value when all are there, compared modulo 2^32).
 // Up to BAR_FEW blocks poll the counter itself (1.19 us per barrier of 152 blocks, 1.31
-// through the flag; a step of 12 cells with 1,216 blocks 484 against 497 us); more
+// through the flag; a step of 12 cells with 608 / 1,216 blocks 418 / 441 us against 441 / 447); more
 // polling blocks hold up the arrivals, so there the last to arrive publishes the target
-// in bar[BAR_FLAG], on another line (2,432 blocks 544 against 719 us, 4,864 blocks 702
-// against 1,070).
+// in bar[BAR_FLAG], on another line (2,432 blocks 464 against 597 us, 4,864 blocks 593
+// against 974).
 // False (and *err raised) if that takes longer than wait_ns nanoseconds or if another
 // block has raised *err.  The clock and the flag are looked at every 32nd poll, at every
 // poll when the limit is below 100 us.
@@ -235,6 +235,30 @@ __device__ __forceinline__ void phase_wall(const CellDesc<T> &c, const Sten<T> s
     if constexpr (CP) c.pl[wb] = (T)0;
 }
 
+// The same wall node by one lane: the partial sums of WALL_LANES lanes side by side, put together
+// in the order of group_sum, so the same bits.
+template <typename T, bool CP>
+__device__ __forceinline__ void phase_wall_one(const CellDesc<T> &c, const Sten<T> st, int64_t b) {
+    static_assert(WALL_LANES == 4, "four sums");
+    if (b >= c.nb) return;
+    const int n_l = c.n_l;
+    const T *p = c.p;
+    T s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+    int j = 1;
+    for (; j + 3 < n_l; j += 4) {
+        s0 += st.wt(j) * p[st.ix(j)];
+        s1 += st.wt(j + 1) * p[st.ix(j + 1)];
+        s2 += st.wt(j + 2) * p[st.ix(j + 2)];
+        s3 += st.wt(j + 3) * p[st.ix(j + 3)];
+    }
+    if (j < n_l) s0 += st.wt(j) * p[st.ix(j)];
+    if (j + 1 < n_l) s1 += st.wt(j + 1) * p[st.ix(j + 1)];
+    if (j + 2 < n_l) s2 += st.wt(j + 2) * p[st.ix(j + 2)];
+    const int32_t wb = c.wall[b];
+    c.p[wb] = -((s0 + s2) + (s1 + s3)) / st.wt(0);
+    if constexpr (CP) c.pl[wb] = (T)0;
+}
+
 // returns |v|^2 of the node (lead lane of a fluid node), 0 otherwise
 template <typename T, bool CP, int G>
 __device__ __forceinline__ T phase_correct(const CellDesc<T> &c, const Sten<T> st, int64_t i, int g, bool valid,
@@ -298,7 +322,7 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
     if constexpr (SH) cells = own; else cells = cells_g;
     double *racc = reinterpret_cast<double *>(own + (SH ? nc : 0));  // [nc][2]
     int64_t *pre = reinterpret_cast<int64_t *>(racc + 2 * nc);  // [nc + 1] units ahead of each cell
-    int64_t *wpre = pre + nc + 1;                               // [nc + 1] wall units
+    int64_t *wpre = pre + nc + 1;                               // [nc + 1] wall slices
     int *done = reinterpret_cast<int *>(wpre + nc + 1);         // [nc]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wpb = blockDim.x >> 5;
@@ -315,7 +339,7 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
         for (int c = threadIdx.x; c < nc; c += blockDim.x) {
             done[c] = 0;
             pre[c + 1] = ((cells_g[c].n + 31) >> 5) * G;
-            wpre[c + 1] = ((cells_g[c].nb + 31) >> 5) * WALL_LANES;
+            wpre[c + 1] = (cells_g[c].nb + 31) >> 5;
         }
     }
     __syncthreads();
@@ -358,13 +382,18 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
             }
         }
     };
+    // Wall nodes by four lanes each while that is one unit a warp; past it one lane per node loses no
+    // time to latency and saves the units' overhead (FP32, 64 cells with 1.6M wall nodes: 5.27 ms
+    // per step against 5.58 with four lanes throughout; FP64, 12 cells 1.12 against 1.14).
+    const int wlog = wpre[nc] * WALL_LANES <= wstride ? 2 : 0;
+    static_assert(WALL_LANES == 4, "1 << wlog");
     auto wall_units = [&](auto &&f) {
         int c = 0;
-        for (int64_t k = k0; k < wpre[nc]; k += wstride) {
-            while (k >= wpre[c + 1]) ++c;
+        for (int64_t k = k0; k < wpre[nc] << wlog; k += wstride) {
+            while (k >= wpre[c + 1] << wlog) ++c;
             if (done[c]) continue;
-            const int64_t un = k - wpre[c];
-            f(cells[c], un / WALL_LANES, (int)(un % WALL_LANES));
+            const int64_t un = k - (wpre[c] << wlog);
+            f(cells[c], un >> wlog, (int)(un & ((1 << wlog) - 1)));
         }
     };
     auto sten = [&](const CellDesc<T> &d, int64_t ls, int nl) {
@@ -417,9 +446,14 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
             });
             if (!barrier()) { broke = true; break; }
             wall_units([&](const CellDesc<T> &d, int64_t ls, int sub) {
-                const int nl = sub * (32 / WALL_LANES) + lane / WALL_LANES;
-                phase_wall<T, CP, WALL_LANES>(d, Sten<T>{d.wn + ((ls * d.n_l) << 5) + nl, d.idxb + ((ls * d.n_l) << 5) + nl},
-                                              (ls << 5) + nl, lane % WALL_LANES);
+                const T *wn = d.wn + ((ls * d.n_l) << 5);
+                const int32_t *ib = d.idxb + ((ls * d.n_l) << 5);
+                if (wlog) {
+                    const int nl = sub * (32 / WALL_LANES) + lane / WALL_LANES;
+                    phase_wall<T, CP, WALL_LANES>(d, Sten<T>{wn + nl, ib + nl}, (ls << 5) + nl, lane % WALL_LANES);
+                } else {
+                    phase_wall_one<T, CP>(d, Sten<T>{wn + lane, ib + lane}, (ls << 5) + lane);
+                }
             });
             if (!barrier()) { broke = true; break; }
             // max |v| of each cell: the largest |v|^2 of this warp's units, one root and one

@@ -1004,8 +1004,8 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
     }
     // Streaming: one lane per node unless asked for otherwise.  More lanes only win while a round
     // of units leaves warps idle (us per step with 256 threads and one lane / 128 and two:
-    // FP32 12 cells 425 / 484, 600k nodes 541 / 597, 113k 181 / 194; FP64 12 cells 1117 / 1317, 24 cells
-    // 1148 / 1150; 15k nodes in 3 cells 108 / 72).
+    // FP32 12 cells 424 / 485, 600k nodes 530 / 577, 6 cells of 113k 168 / 192; FP64 12 cells 1118 / 1304,
+    // 24 cells 1149 / 1130; FP32 15k nodes in 3 cells 106 / 67).
     p.block = x->persist_block ? x->persist_block : 256;
     p.group = x->persist_block ? x->persist_group : 1;
     int64_t slices = 0;

@@ -128,21 +128,23 @@ def test_descriptor_copies_change_nothing(prec):
 
 
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
-def test_one_lane_solve_equals_the_step_kernels(prec):
-    """Code 256 of both: the same sums in the same order, so the same bits."""
+@pytest.mark.parametrize("n_axis,n_l", [(14, 25), (29, 24)])
+def test_one_lane_solve_equals_the_step_kernels(prec, n_axis, n_l):
+    """Codes of one lane per node: the same sums in the same order, so the same bits, with the wall nodes by four
+    lanes each (the grid; the smaller cell on a cluster of 64 warps) and by one (1,295 of them on the cluster)."""
     rbf = gpu_or_skip()
-    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=14, seed=5))
+    s = _solver(rbf, synth.jittered_cell(r=0.35, n_axis=n_axis, seed=5), n_l)
     got = []
-    for solve in (0, 1):
+    for code in (None, 256, -8):
         s.init(precision=rbf.RBF_FP64 if prec == "fp64" else rbf.RBF_FP32, v_ref=0.01)
-        if solve:
-            s.set_persistent_block(256)
+        if code:
+            s.set_persistent_block(code)
             s.solve(40, 1e-300)
         else:
             s.set_kernel_variant(256)
             s.step(40)
         got.append(s.get_fields())
-    assert np.abs(got[0]).max() > 0 and np.array_equal(*got)
+    assert np.abs(got[0]).max() > 0 and all(np.array_equal(g, got[0]) for g in got[1:])
     s.close()
 
 
