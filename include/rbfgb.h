@@ -109,7 +109,9 @@ typedef struct {
 /* RBF-FD weights, Eqs. operatorApprox, rbfScaling and augmentedSystem: PHS
  * r^phs_k (odd, >= 3) in the distance scaled by delta_i (distance from x_i to its
  * nearest neighbour), augmented with the C(mono_m + 3, 3) monomials of degree
- * <= mono_m; solved per node in FP64 by LU with partial pivoting.
+ * <= mono_m; solved per node to FP64: r^3 and r^5 by an FP32 inverse refined with
+ * residuals of the FP64 system, the few systems where that does not converge and r^7
+ * and up by LU with partial pivoting and one refinement.
  *  solver RBF_SOLVER_ACM: d/dx, d/dy, d/dz, Laplacian at every node, plus the
  *         gradient on every wall node's Neumann stencil.
  *  solver RBF_SOLVER_LBM: interpolation to the departure points x_i - dx e_k

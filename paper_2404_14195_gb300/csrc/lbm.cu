@@ -360,7 +360,7 @@ __device__ __forceinline__ void step_records(const LbmArgs<T> &a, int64_t first)
 // beat one column at 64 registers and 32 warps: the bytes in flight are the same, but a
 // wave holds half the nodes and a thread waits half as often.  Measured (us per step, D3Q19,
 // N_L = 30; in brackets one column at 64 registers, and the time of the bytes at the copy
-// bandwidth): 71k nodes 27.5 (32.1, 25.5), 152k 54.9 (57.4, 54.5), 172k 67.1 (94.4, its 672
+// bandwidth, of which 2 % do not leave the L2): 71k nodes 27.5 (32.1, 25.5), 152k 54.9 (57.4, 54.5), 172k 67.1 (94.4, its 672
 // blocks left a nearly empty second wave; 61.6), 261k 102.5 (113, 93.5).
 // FP64 is bound by its pipe (2 lanes per clock and SM): 172k nodes 262 us, 216 for the
 // products alone; the pairs schedule, whose moments every pair repeats, 496.

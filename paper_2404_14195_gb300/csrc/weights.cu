@@ -10,7 +10,8 @@
 //   b_j = (L Phi_j)(y), c_l = (L p_l)(y),  y = x_c + off
 // either from an FP32 inverse refined to FP64 (k <= 5, k_weights_fast) or by an FP64 LU with
 // partial pivoting and one refinement (k_weights: k >= 7, and the systems that the first one
-// hands on).  Residuals are exact in both.  delta is the distance to the nearest other node
+// hands on).  Residuals are formed in integers in both; row_products and Residual32 say what
+// they drop.  delta is the distance to the nearest other node
 // (centre is a node) or to the nearest node (centre is a free point such as a permeability
 // probe).
 //
@@ -19,7 +20,7 @@
 //  * The residual, which has to carry about twice the working precision, runs on
 //    the integer pipe: rows of M and columns of x are cut into three 26/27-bit
 //    slices relative to the row's (column's) largest exponent, six to eight 32 x 32 -> 64
-//    bit multiply-adds per product accumulate exactly.  A compensated FP64 dot product (ten
+//    bit multiply-adds per product accumulate without rounding.  A compensated FP64 dot product (ten
 //    FP64 operations per product) was two thirds of the FP64 work of an 18-operator system.
 //  * One reciprocal per pivot instead of a division per right-hand side; each
 //    distance of the symmetric A computed once.
@@ -29,7 +30,7 @@
 //    buffers are reused, which leaves 4-5 blocks (16-20 warps) per SM at N_L = 30..40.
 // Measured (GB300, 2070 MHz), 86,397 systems of n = 60 with 4 operators (N_L = 40, r^5,
 // m = 3) / 120,840 systems of n = 40 with 18 operators (N_L = 30, r^3, m = 2): FP32 inverse
-// 19 / 24 ms, with no pipe above 75 % (integer multiplies 54 / 71 %, FP64 38 / 23 %); FP64 LU
+// 19 / 24 ms, with no pipe above 75 % (integer multiplies 50 / 60 %, FP64 43 / 29 %); FP64 LU
 // 34.4 / 33.5 ms, the FP64 pipe 81-87 % busy; one warp per system with FP64 LU and the
 // compensated product 164 / 167 ms.
 #include <algorithm>
@@ -145,8 +146,9 @@ __device__ __forceinline__ double pow2(int e) {  // 2^e, clamped to the normal r
 // Products of row r of M0 with NO columns of X (operators o0, o0 + step, ...): the 80-bit
 // fixed-point slices of both give eight 32 x 32 -> 64 bit products per entry, whose sums fit 64
 // bits (ns <= 99: T0 < 2^59, T1 < 2^61, T2, T3 < 2^62); T0 counts 2^108, T1 2^81, T2 2^54, T3
-// 2^27 units of 2^(er + ex - 2204).  Only terms below 2^-108 of (row maximum) x (column
-// maximum) are dropped.
+// 2^27 units of 2^(er + ex - 2204).  Of (row bound) x (column bound) a product drops 2^-106, and
+// what cut() leaves off an operand more than 2^-27 below its bound, at most 2^-80 each: below
+// ns 2^-79 in all, 2^-72 for the largest system.
 template <int NO>
 __device__ __forceinline__ void row_products(int r, int ns, int n_ops, int o0, int step, int er, const double *M0,
                                              const int4 *Xs, long long (&t0)[NO], long long (&t1)[NO],
@@ -516,7 +518,7 @@ __device__ void weights_fp64(int64_t c, double *sm, const WJob &J) {
 // The same systems by an FP32 inverse and iterative refinement to FP64: the residual is formed
 // in integers, each correction is the FP32 inverse times it, and x in FP64 converges to the
 // solution of the stored FP64 system, as the refinement of the FP64 factors does.  The
-// componentwise condition numbers of stencil systems are 1e2 .. 1e5 (PHS r^3, r^5), so a
+// componentwise condition numbers of stencil systems are mostly 1e2 .. 1e5 (PHS r^3, r^5), so a
 // correction gains 3 to 4 digits.  An operator is done when what its last correction (from a
 // full residual) leaves, that times the ratio of the last two, is below 2^-56 of its largest
 // weight.  A system whose pivot falls below 1e-5 of its row, or that has not converged after MAX_ITER
@@ -558,7 +560,8 @@ constexpr int MAX_ITER = 12;
 // and RT CT multiply-adds for RT + CT loads.
 //
 // Row i of the tile to shared memory, with 1 in the column of elimination (at: its thread),
-// and zeroed.  The comment keeps the branches of the rows apart: merged, they index the tile.
+// and zeroed.  The comment keeps the branches of the rows apart: merged, they would index the
+// tile, which then lives in local memory (a matter of speed only).
 template <int RT, int CT, int I>
 __device__ __forceinline__ void put_row(int i, bool at, float (&a)[RT][CT], float *row) {
     if (i == I) {
@@ -769,9 +772,15 @@ __device__ __noinline__ float difference(double B, long long t0, long long t1, l
 }
 
 // Rf <- B - M0 X as multiples of 2^(ex - 1022) (about the size of X's column), in integers up
-// to the conversion.  FULL: all products above 2^-80 of (row maximum) x (column maximum), with
-// which 1e6 in condition still leaves the last bits right.  Otherwise those above 2^-53, all
-// that the first x needs.
+// to the conversion.  FULL: three levels of slice products; what is dropped (two products below
+// 2^-79 of (row bound) x (column bound) per term, and what cut() leaves off small operands) stays
+// below ns 2^-77.4, 2^-71 for the largest system.  Times a componentwise condition of 1e5 that is
+// 2^-54 of the operator's largest weight at worst (2^-48 for the worst r^5 systems of 64 nodes,
+// 6e6).  Measured against 113-bit arithmetic over N_L = 20 .. 64 (r^3 and r^5, 1,300 systems): the
+// root mean square error is 25 % below that of FP64 LU with one compensated refinement, the
+// largest error of a weight relative to itself at or below it, and that of weights below 1e-4 of the
+// largest as well (the rounding of the stored matrix decides all of them).  Otherwise two levels,
+// 2^-53: all that the first x needs.
 template <bool FULL>
 struct Residual32 : Fast {
     template <int NO>
