@@ -61,9 +61,9 @@ R, H_MIN, H_MAX, RAMP, SEED = 0.40, 0.008, 0.04, 0.2, 2
 N_L, Q, DX, TAU_P, MAGIC = 30, 19, 0.004, 0.8, 3.0 / 16.0
 KERNELS = {0: "k_lbm_step<float,19> (256)", 1: "k_lbm_step_pairs<float,19,5>", 2: "k_lbm_step<float,19> (128)",
            3: "k_lbm_step_pairs<float,19,3>", 4: "k_lbm_step_pairs<float,19,6>", 5: "k_lbm_step_pairs<float,19,2>",
-           6: "k_lbm_step_records<float,19,4> (256)", 7: "k_lbm_step_records<float,19,5> (256)",
-           8: "k_lbm_step_records<float,19,4> (128)", 9: "k_lbm_step_records<float,19,4> (64)",
-           10: "k_lbm_step_records<float,19,4,PDL> (256)"}
+           6: "k_lbm_step_records<float,19,2,1> (256)", 7: "k_lbm_step_records<float,19,5,1> (256)",
+           8: "k_lbm_step_records<float,19,2,1> (128)", 9: "k_lbm_step_records<float,19,2,1> (64)",
+           10: "k_lbm_step_records<float,19,2,1,PDL> (256)"}
 
 
 def workload():
@@ -354,8 +354,8 @@ def main():
     # the residual (4 B per population)
     bpl = (bytes_per_node_step(elt=elt) + (4 * Q if args.precision == "fp32r" else 0)) * n
     achieved = bpl / (per_launch_ms / 1e3) / 1e9
-    kname = KERNELS[chosen] if elt == 4 else (KERNELS[chosen].replace("float", "double")
-                                              .replace(",19,4>", ",19,2>").replace(",19,5>", ",19,3>"))
+    kname = KERNELS[chosen] if elt == 4 else (KERNELS[chosen].replace("float", "double").replace(",19,5,", ",19,3,")
+                                              .replace("PDL> (256)", "PDL> (64)"))
     cpu = None if (args.no_cpu_baseline or ws > 1) else oracle_baseline(case)
     refs = golden_references()
     tts = None
