@@ -1116,6 +1116,7 @@ bool acm_resident_plan(int64_t n, int64_t nb, int n_l, int group, int sms, int64
     pl->nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(sms, units));
     const int64_t u = (units + pl->nblocks - 1) / pl->nblocks, wu = (wunits + pl->nblocks - 1) / pl->nblocks;
     if (u * nu * n_l * 4 * (int64_t)sizeof(T) > room) return false;
+    pl->room = (int)room;
     pl->units = (int)u;
     pl->wunits = (int)wu;
     pl->loc = 0;
@@ -1136,9 +1137,7 @@ cudaError_t acm_launch_resident(const CellDesc<T> &cell, const PersistCtl &ctl, 
     const void *fn = cp ? resident_kernel<T, true>(group) : resident_kernel<T, false>(group);
     if (block < 32 || block % 32 || block > (sizeof(T) == 4 ? 1024 : 512) || !fn) return cudaErrorInvalidValue;
     // the kernel's limit is one for all threads of the program: always the same value
-    int room = 0;
-    cudaError_t e = resident_room(&room);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, room);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.room);
     if (e != cudaSuccess) return e;
     void *args[] = {(void *)&cell, (void *)&ctl, (void *)&pl};
     return cudaLaunchCooperativeKernel(fn, dim3(pl.nblocks), dim3(block), args, (size_t)pl.smem, st);

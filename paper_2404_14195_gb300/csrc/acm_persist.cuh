@@ -66,18 +66,10 @@ constexpr int64_t persist_head_bytes(int ncells, bool shared) {
 }
 // Shares of the resident kernel (one cell, every block's stencils in shared memory):
 // largest number of units and wall units per block, local nodes there is room for,
-// dynamic shared memory, blocks.
+// dynamic shared memory, blocks; room: what a block may take.
 struct ResPlan {
-    int units, wunits, loc, smem, nblocks;
+    int units, wunits, loc, smem, nblocks, room;
 };
-// dynamic shared memory that a block of the resident kernel may take on the current device
-inline cudaError_t resident_room(int *room) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(room, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    *room -= 2048;
-    return e;
-}
 // whether a cell can run resident with `room` bytes of shared memory on each of `sms` SMs (its
 // local sets are only known to the kernel, which raises error 3 before the first step if one has
 // no room)

@@ -355,6 +355,7 @@ int rbf_create(rbf_ctx **out, int device, void *cuda_stream) {
         ctx->own_stream = true;
     }
     if (cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&ctx->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess ||
         cudaEventCreate(&ctx->ev0) != cudaSuccess || cudaEventCreate(&ctx->ev1) != cudaSuccess ||
         ctx->vmax.alloc(2) != cudaSuccess || ctx->scal.alloc(16) != cudaSuccess || ctx->status.alloc(4) != cudaSuccess ||
         static_flux_lookup(&ctx->static_flux) != cudaSuccess) {
@@ -985,18 +986,14 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
         p.csize = p.nblocks = x->persist_cluster;
         return p;
     }
-    int sms = 0, room = 0;
-    p.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, x->device);
-    if (p.err == cudaSuccess) p.err = resident_room(&room);
-    if (p.err != cudaSuccess) return p;
     // One cell whose shares fit runs resident, unless one lane per node was asked for (which
     // keeps the summation order of the multi-launch kernels).
     if (cs.size() == 1 && (!x->persist_block || x->persist_group > 1)) {
         p.group = x->persist_group;
-        if (!x->persist_block) resident_auto(x->n / (double)sms, sizeof(T) == 8, &p.block, &p.group);
+        if (!x->persist_block) resident_auto(x->n / (double)x->sms, sizeof(T) == 8, &p.block, &p.group);
         else p.block = std::min<int>(sizeof(T) == 4 ? 1024 : 512, std::max<int>(x->persist_block, 256));
         p.resident = !(x->res_nofit & res_bit<T>(p.group)) &&
-                     acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, sms, room, &p.res);
+                     acm_resident_plan<T>(x->n, x->nb, x->n_l, p.group, x->sms, x->smem_optin - 2048, &p.res);
         if (p.resident) {
             p.nblocks = p.res.nblocks;
             return p;

@@ -43,7 +43,7 @@ struct DevArr {
 
 struct rbf_ctx {
     template <typename T> using DevArr = rbf::DevArr<T>;
-    int device = 0, sms = 1;
+    int device = 0, sms = 1, smem_optin = 0;  // SMs, shared memory a block may ask for
     cudaStream_t st = nullptr;
     bool own_stream = false;
     std::string err;
