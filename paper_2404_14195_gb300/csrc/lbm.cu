@@ -195,9 +195,12 @@ template <> struct Vec2<float> { using type = float2; };
 template <> struct Vec2<double> { using type = double2; };
 
 // One thread per node: all q populations of the node in registers.  RA: add the
-// residual a.radd to the post-collision populations (refined FP32).
+// residual a.radd to the post-collision populations (refined FP32).  The blocks per SM are stated
+// because without them the compiler stops at 40 registers (FP64: 66) and asks for the columns'
+// loads one after the other (D3Q15 FP32, blocks of 128: 121k nodes 70 us per step, 47 at 64
+// registers; 16k nodes 55, 20).
 template <typename T, int Q, bool RA = false>
-__global__ void __launch_bounds__(256) k_lbm_step(LbmArgs<T> a) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_lbm_step(LbmArgs<T> a) {
     using V = typename Vec2<T>::type;
     constexpr int NP = (Q - 1) / 2;
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
