@@ -266,7 +266,7 @@ int rbf_profile_steps(rbf_ctx *ctx, int nsteps, double *kernel_ms, int *n_classe
  * blocks by the size of the grid, a grid that fills the chip launched as a
  * programmatic dependent launch (the next step's blocks are scheduled while this
  * step drains and wait on the grid dependency before touching memory).  Until a
- * code is set: 10, cells below 4096 nodes 1.
+ * code is set: 10, small cells 1 (by nodes per SM, precision and q).
  * Switching between the two layouts on an initialised LBM
  * context rewrites the state (one kernel launch); the populations, as
  * rbf_lbm_get_populations reports them, are unchanged.

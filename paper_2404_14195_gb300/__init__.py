@@ -349,7 +349,7 @@ class Solver:
         4 or 8 lanes per node) with 256 / 128 / 64 threads per block; 7 one node
         per thread with registers capped for more blocks per SM; 10 as 6 with
         blocks by the size of the grid, large grids as programmatic dependent
-        launches (the default, cells below 4096 nodes 1).  The state is
+        launches (the default, small cells 1).  The state is
         rewritten when the layout changes.
         ACM (after compute_weights for the ACM): threads per block (64, 128,
         256) + 1000 x lanes per node (2, 4; 0 for one) of the step sweeps."""

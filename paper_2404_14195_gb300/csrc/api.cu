@@ -727,6 +727,27 @@ int rbf_get_weights(rbf_ctx *ctx, int op, double *out) {
     return RBF_OK;
 }
 
+// The LBM schedule until one is set: node records, except where a pair per warp is faster, by nodes
+// per SM.  It spreads a node over (q - 1) / 2 warps, which wins on small cells, longer in FP32 and
+// with D3Q15, which has fewer sums to split.  us per step of a graph, pair per warp / node records:
+//   FP32 D3Q15  5k nodes 4.4 / 6.1, 14k 6.9 / 8.1, 24k 10.9 / 13.1, 31k 15.3 / 14.2, 66k 24.8 / 21.2
+//        D3Q19  5k 5.4 / 7.6, 9k 7.4 / 7.9, 14k 10.6 / 10.4, 18k 13.3 / 11.1
+//   FP64 D3Q15  5k 19.3 / 22.0, 9k 24.0 / 20.8; D3Q19 2k 18.8 / 27, 5k 27.2 / 26.7, 9k 33.6 / 26.2
+// D3Q15 FP32 past the small cells: the records' time goes with the blocks of 256 on the fullest SM,
+// the pairs', 10 % more per node, with the nodes, so where that last block is mostly missing the
+// pairs win (2.1 to 5.5 blocks per SM: 81k 29.3 / 34.2, 96k 33.7 / 34.4, 103k 35.4 / 34.4, 127k 41.8 /
+// 43.7, 152k 49.4 / 44.1, 168k 53.4 / 54.8, 180k 57.0 / 55.2, 198k 61.1 / 64.2, 214k 65.8 / 64.8).
+static int lbm_variant_by_size(int64_t n, int sms, int q, bool fp64) {
+    const double per = (double)n / sms;
+    bool pairs;
+    if (fp64) pairs = per < (q == 15 ? 40.0 : 27.0);
+    else if (q == 15) {
+        const double b = per / 256.0;
+        pairs = per < 170.0 || (b > 1.75 && b < 6.0 && 1.1 * b + 0.24 < std::ceil(b));
+    } else pairs = per < 66.0;
+    return pairs ? LBM_PAIR_PER_WARP : LBM_RECORD_PER_THREAD_PDL;
+}
+
 int rbf_init(rbf_ctx *ctx, const rbf_params *p) {
     if (!ctx || !p) return RBF_EINVAL;
     if (!ctx->weights_ok) return fail(ctx, RBF_EINVAL, "rbf_init: compute weights first");
@@ -776,10 +797,7 @@ int rbf_init(rbf_ctx *ctx, const rbf_params *p) {
         ctx->dt = ctx->lbm_dt;
         for (int a = 0; a < 3; ++a) ctx->gl[a] = p->g[a] * ctx->lbm_dt * ctx->lbm_dt / ctx->dx;
         ctx->cur = 0;
-        // Until a schedule is set: node records, except for the smallest cells, where a pair per
-        // warp spreads a node over nine warps (1.7k nodes: FP64 13.4 us per step against 17.5, FP32
-        // 4.4 against 4.6; 6k nodes: 33.7 against 29.9, 6.9 against 7.2)
-        if (ctx->variant_auto) ctx->variant = n < 4096 ? LBM_PAIR_PER_WARP : LBM_RECORD_PER_THREAD_PDL;
+        if (ctx->variant_auto) ctx->variant = lbm_variant_by_size(n, ctx->sms, ctx->q, ctx->prec == RBF_FP64);
         ctx->lbm_layout = lbm_layout_of(ctx->variant);
         const int64_t sz = (int64_t)lbm_rec_len(ctx->q) * npad;  // room for either layout
         if (ctx->prec == RBF_FP32R) {

@@ -603,8 +603,10 @@ static cudaError_t launch_records_k(const LbmArgs<T> &a, cudaStream_t st, int bl
 // as many lanes as keep the threads per SM below a limit: FP32 280 (21k nodes: 2 lanes 13.0 us
 // per step, 4 lanes 18.2, 1 lane 15.6; 6k: 4 lanes 7.2, 8 lanes 8.1), FP64 160, because the
 // lanes of a node repeat its collision on the pipe that is the bound (21k: 1 lane 49.4, 2
-// lanes 62; 6k: 4 lanes 29.9, 1 lane 36.0).  block = 0: 64 threads while the grid is small
-// (finer pieces spread more evenly), else 256; FP64 64.  FP64 cells past 320 nodes per SM have
+// lanes 62; 6k: 4 lanes 29.9, 1 lane 36.0).  block = 0: 64 threads until blocks of 256
+// nearly fill the SMs twice (finer pieces spread more evenly: FP32 D3Q15 50k nodes 20.5 us against
+// 24.7, 66k 22.7 against 24.7, D3Q19 22.7 against 26.9 and 28.5 against 28.7; 73k 26.6 against 24.7
+// and 32.4 against 29.4), then 256; FP64 64.  FP64 cells past 320 nodes per SM have
 // the warps to hide the latency and run one column at a time in 128 registers (121k: 191 us
 // against 199).
 template <typename T, int Q, bool RA, bool PDL>
@@ -613,7 +615,7 @@ static cudaError_t launch_records(const LbmArgs<T> &a, cudaStream_t st, int bloc
     constexpr int MB = D ? 1 : 2;
     int lanes = 1;
     while (lanes < 8 && a.n * lanes * 2 <= (int64_t)a.sms * (D ? 160 : 280)) lanes *= 2;
-    if (block == 0) block = D || a.n * lanes < (int64_t)a.sms * 320 ? 64 : 256;
+    if (block == 0) block = D || a.n * lanes < (int64_t)a.sms * 448 ? 64 : 256;
     if constexpr (D) {
         if (a.n > (int64_t)a.sms * 320) return launch_records_k<T, Q, 2, 1, RA, PDL, false, 1>(a, st, block);
     }
