@@ -321,7 +321,8 @@ int rbf_autotune_persistent(rbf_ctx *ctx, int trial_steps, rbf_tune_report *rep)
  *   -8, -16          one cluster of 8 / 16 CTAs of 256 threads, G = 1;
  *   0                chosen by the size of the cells, as until a code is set: one cell
  *                    whose stencils fit resident with 1, 2 or 4 lanes per node and 256
- *                    or 512 threads, everything else as 256.
+ *                    or 512 threads, everything else as 256 or, in FP64 with a short
+ *                    round of work left over, as 2128.
  * A batch launches with its first cell's setting.  With G = 1 the schedule
  * changes only the order of the FP64 residual partial sums; G > 1 also changes
  * the order of the stencil sums (rounding only). */

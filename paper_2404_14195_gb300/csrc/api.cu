@@ -1017,16 +1017,26 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
             return p;
         }
     }
-    // Streaming: one lane per node unless asked for otherwise.  More lanes only win while a round
-    // of units leaves warps idle (us per step with 256 threads and one lane / 128 and two:
-    // FP32 12 cells 424 / 485, 600k nodes 530 / 577, 6 cells of 113k 168 / 192; FP64 12 cells 1118 / 1304,
-    // 24 cells 1149 / 1130; FP32 15k nodes in 3 cells 106 / 67).
+    // Streaming: one lane per node unless asked for otherwise, two in FP64 where a short round would
+    // be left over, whose few warps on each SM's pipe take the time of some 0.4 rounds at one lane and
+    // half of that at two.  us per step with 256 threads and one lane / 128 and two:
+    //   FP64, rounds of one-lane units 1.10: 477 / 453, 1.12: 526 / 497, 1.20: 486 / 438, 1.33: 529 / 491,
+    //   2.19: 827 / 753, 3.16: 1148 / 1130; 0.98: 384 / 402, 1.78: 586 / 614, 1.82: 460 / 533, 4.00: 1118 / 1304
+    //   FP32 12 cells 424 / 485, 600k nodes 530 / 577, 6 cells of 113k 168 / 192
     p.block = x->persist_block ? x->persist_block : 256;
     p.group = x->persist_block ? x->persist_group : 1;
     int64_t slices = 0;
     for (const rbf_ctx *y : cs) slices += y->npad / 32;
     int maxb = 0;
     p.err = acm_persistent_max_blocks<T>(&maxb, p.block, p.group, cp, (int)cs.size());
+    if (sizeof(T) == 8 && !x->persist_block && p.err == cudaSuccess) {
+        const double rounds = slices / (8.0 * maxb), over = rounds - std::floor(rounds);
+        if (rounds > 1.0 && rounds < 4.0 && over > 0.04 && over < 0.4) {
+            p.block = 128;
+            p.group = 2;
+            p.err = acm_persistent_max_blocks<T>(&maxb, p.block, p.group, cp, (int)cs.size());
+        }
+    }
     const int64_t wpb = p.block / 32, units = slices * p.group;
     p.nblocks = (int)std::max<int64_t>(1, std::min<int64_t>(maxb, (units + wpb - 1) / wpb));
     return p;

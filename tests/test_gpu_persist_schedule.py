@@ -84,26 +84,25 @@ def test_streaming_blocks_per_sm():
     s.close()
 
 
-@pytest.mark.parametrize("prec", ["fp64", "fp32", "fp32c"])
-def test_batch_default_is_one_lane_per_node(prec):
-    """24 cells, about 12,300 units: 3.4 rounds of an FP64 grid's 3,648 warps, 2.5 of an FP32 grid's
-    4,864.  One lane per node, and the same fields from blocks of 32 threads."""
+@pytest.mark.parametrize("prec,n_cells,lanes", [("fp64", 24, 2), ("fp64", 28, 1), ("fp32", 24, 1), ("fp32c", 24, 1)])
+def test_batch_default_lanes(prec, n_cells, lanes):
+    """About 510 units a cell.  FP64 grids hold 3,648 warps: 24 cells leave a short round over (3.4 rounds) and take
+    two lanes per node, 28 cells (3.9) one; FP32 always one.  The same fields from blocks of 32 threads."""
     rbf = gpu_or_skip()
     b = rbf.Batch(0)
-    cells = [synth.jittered_cell(r=0.3, n_axis=25 + i % 3, seed=40 + i) for i in range(24)]
-    for c in cells:
-        b.add_cell(c, 20)
+    for i in range(n_cells):
+        b.add_cell(synth.jittered_cell(r=0.3, n_axis=25 + i % 3, seed=40 + i), 20)
     b.build(3, 2)
     p = {"fp64": rbf.RBF_FP64, "fp32": rbf.RBF_FP32, "fp32c": rbf.RBF_FP32C}[prec]
     got = []
-    for code in (None, 32):
+    for code in (None, 32 if lanes == 1 else 1000 * lanes + 32):
         if code:
             b.set_persistent_block(code)
         b.init(precision=p, v_ref=0.01)
-        assert [r["steps"] for r in b.solve(6, 1e-300, check_every=3)] == [6] * 24
+        assert [r["steps"] for r in b.solve(6, 1e-300, check_every=3)] == [6] * n_cells
         i = b.cell(0).persistent_info()
-        assert i["lanes"] == 1 and i["threads"] == (code or 256) and not i["resident"]
-        got.append([b.cell(j).get_fields() for j in range(24)])
+        assert i["lanes"] == lanes and not i["resident"] and i["threads"] == (32 if code else 256 // lanes)
+        got.append([b.cell(j).get_fields() for j in range(n_cells)])
     for x, y in zip(*got):
         assert np.abs(x).max() > 0 and np.array_equal(x, y)
 
