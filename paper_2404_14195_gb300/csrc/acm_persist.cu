@@ -353,9 +353,11 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
     __syncthreads();
     const int64_t wstride = (int64_t)nblocks * wpb, k0 = (int64_t)blockIdx.x * wpb + warp;
 
-    // FP64 is bound by each SM's own pipe, so there the units left over after whole rounds are dealt
-    // out to the blocks in turn (a quarter round on a few SMs costs a whole one: 24 cells, 3.2
-    // rounds 1.24 -> 1.15 ms per step); in FP32 they stay in order, next to each other.
+    // FP64 is bound by each SM's own pipe, so there the units of several lanes per node that are left
+    // over after whole rounds are dealt out to the blocks in turn (a quarter round on a few SMs costs
+    // a whole one: 9 cells, 4.4 rounds of two lanes 812 -> 753 us per step); in FP32 they stay in
+    // order, next to each other, and at one lane too (20k nodes FP64 169 us dealt out, 155 in order; the
+    // default takes two lanes where a short round would be left over).
     auto dealt = [&](int64_t total, auto &&f) {
         const int64_t whole = total < wstride ? total : total - total % wstride;
         const int64_t last = whole + (int64_t)warp * nblocks + blockIdx.x;
@@ -366,7 +368,7 @@ __global__ void __launch_bounds__(256, CL ? 1 : persist_warps<T>() / 8) k_acm_pe
     // descriptor, slice, unit of the slice)
     auto units = [&](auto &&f) {
         int c = 0;
-        if constexpr (sizeof(T) == 8) {
+        if constexpr (sizeof(T) == 8 && G > 1) {
             dealt(pre[nc], [&](int64_t k) {
                 while (k >= pre[c + 1]) ++c;
                 if (done[c]) return;

@@ -1020,8 +1020,8 @@ PersistPlan persist_plan(const std::vector<rbf_ctx *> &cs, bool cp) {
     // Streaming: one lane per node unless asked for otherwise, two in FP64 where a short round would
     // be left over, whose few warps on each SM's pipe take the time of some 0.4 rounds at one lane and
     // half of that at two.  us per step with 256 threads and one lane / 128 and two:
-    //   FP64, rounds of one-lane units 1.10: 477 / 453, 1.12: 526 / 497, 1.20: 486 / 438, 1.33: 529 / 491,
-    //   2.19: 827 / 753, 3.16: 1148 / 1130; 0.98: 384 / 402, 1.78: 586 / 614, 1.82: 460 / 533, 4.00: 1118 / 1304
+    //   FP64, rounds of one-lane units 1.12: 608 / 493, 1.20: 536 / 437 and 415 / 450, 2.19: 951 / 753,
+    //   3.17: 1238 / 1137; 0.96: 236 / 287, 4.00: 1112 / 1306
     //   FP32 12 cells 424 / 485, 600k nodes 530 / 577, 6 cells of 113k 168 / 192
     p.block = x->persist_block ? x->persist_block : 256;
     p.group = x->persist_block ? x->persist_group : 1;
